@@ -169,6 +169,34 @@ int gemm_lmhead_blocks(int vocab);  // number of 256-column partial records per 
 bool encode_tmap(CUtensorMap* tm, CUtensorMapDataType dt, int rank, void* ptr, const uint64_t* dims,
                  const uint64_t* strides, const uint32_t* box, CUtensorMapSwizzle swizzle);
 
+// ---------------------------------------------------------------- few-row GEMM (gemm_few.cu)
+// out = X[M][K] @ W[N][K]^T for at most FEW_MAX_ROWS rows, weight rows on the MMA's M side
+// and the rows of X on its N side; epilogues EPI_BF16, EPI_RESID_F32, EPI_QKV_ROPE, EPI_SWIGLU.
+constexpr int FEW_MAX_ROWS = 128;
+struct FewEpi {
+  void* out = nullptr;             // as EpiParams::out (with QKV: q, and k / v without the stores below)
+  int ldo = 0;
+  const float2* rope = nullptr;    // {cos, sin} [positions][head_dim / 2]
+  int rope_cols = 0, head_dim = 0, k_col0 = 0;
+  __nv_bfloat16* kdst = nullptr;   // QKV: key store [batch][T][G * head_dim] (NULL: k columns of out)
+  __half* vdst = nullptr;          // QKV: v^T store [batch * G][head_dim][Tp] (NULL: v columns of out)
+  int G = 0, T = 0, Tp = 0;
+  const int* m_dev = nullptr;      // device row count (<= M), or NULL
+  const int* row_pos = nullptr;    // QKV: position and sequence of each row
+  const int* row_seq = nullptr;
+  int w_early = 0;                 // 1: the weights may be read before the dependent-launch wait
+};
+struct FewPlan {
+  CUtensorMap tw, tx;
+  int M = 0, N = 0, K = 0, epi = EPI_BF16;
+  int nt_max = 0;  // the rows a launch may hold: 32 or FEW_MAX_ROWS (fewer give a deeper ring)
+  int units = 0, split = 1;  // tiles of 128 weight rows, CTAs (a cluster) that share a tile's K
+  FewEpi ep;
+};
+cudaError_t few_plan(FewPlan* plan, const void* X, int M, int K, const void* W, int N, int epi, const FewEpi& ep,
+                     int num_sms, int nt_max);
+cudaError_t few_launch(const FewPlan& plan, int* err, cudaStream_t stream);
+
 // ---------------------------------------------------------------- attention (attention_tc.cu)
 // softmax(q k^T / sqrt(hd)) v per (sequence, head): the query rows of sequence b are rows
 // [seq_off[b], seq_off[b] + seq_len[b]) of qkv (q columns) and of out (NULL tables: b*T and
@@ -216,14 +244,23 @@ struct RowPlan {
 // current block).  update = 0 plans the rows without recording the prefix end (a forward
 // that commits nothing, e.g. a debug pass, leaves the next step's refresh decision
 // unchanged).
+// select: the conditional node that takes the step's branch (StepBranch of the row count), or 0.
 cudaError_t row_plan_launch(const RowPlan& rp, const int32_t* p, int batch, int N, int T, int block_len,
-                            int cached, int update, int32_t* x, int window, int mask_id, cudaStream_t stream);
+                            int cached, int update, int32_t* x, int window, int mask_id,
+                            cudaGraphConditionalHandle select, cudaStream_t stream);
+// The GEMM kernels of a step, by the rows it computes.
+enum StepBranch : int { STEP_PAIR = 0, STEP_FEW32 = 1, STEP_FEW = 2, STEP_BRANCHES = 3 };
+__host__ __device__ inline int step_branch(int rows) {
+  return rows <= 32 ? STEP_FEW32 : rows <= FEW_MAX_ROWS ? STEP_FEW : STEP_PAIR;
+}
 cudaError_t embed_remask_launch(int32_t* x, const int32_t* p, int batch, int T, int window,
                                 int mask_id, int vocab, const __nv_bfloat16* embed, int d,
                                 float* h, int* err, const RowPlan& rp, cudaStream_t stream);
-// y row r = normalised x row src[r] (src NULL: r), for r < min(rows, *rows_dev).
+// y row r = normalised x row src[r] (src NULL: r), for r < min(rows, *rows_dev).  early: let the
+// next kernel be scheduled before this one's dependent-launch wait (a few-row GEMM, which then
+// fills its ring with weights while this kernel and the one before it run).
 cudaError_t rmsnorm_launch(const float* x, const __nv_bfloat16* gain, __nv_bfloat16* y, int rows,
-                           int d, float eps, const int* rows_dev, const int* src, cudaStream_t stream);
+                           int d, float eps, const int* rows_dev, const int* src, bool early, cudaStream_t stream);
 // Per-position outputs of the softmax statistics (any pointer but top1 may be NULL).
 struct ConfOut {
   int32_t* top1 = nullptr;
@@ -269,7 +306,8 @@ cudaError_t generate_launch(__nv_bfloat16* dst, uint64_t seed, int tid, int64_t 
                             int blk_stride, int blk_off, cudaStream_t stream);
 // cos / sin of the rotate-half angles t * theta^(-2j/hd), computed in double on the host,
 // laid out [hd/2][T] (positions contiguous).
-cudaError_t rope_table_build(float* cos_dev, float* sin_dev, int T, int hd, float theta,
+// cs_dev: the same as {cos, sin} [T][hd/2].
+cudaError_t rope_table_build(float* cos_dev, float* sin_dev, float2* cs_dev, int T, int hd, float theta,
                              cudaStream_t stream);
 
 // Message returned by dcl_last_error(NULL) for calls that have no context.

@@ -30,6 +30,12 @@ struct Launch {  // one kernel launch of the step, for profiling
   cudaEvent_t start, stop;
 };
 
+struct ProfGraph {  // a step graph with timing events around every kernel
+  cudaGraphExec_t exec = nullptr;
+  std::vector<Launch> launches;
+  size_t n = 0;  // launches of the graph
+};
+
 }  // namespace
 
 struct dcl_ctx {
@@ -70,6 +76,7 @@ struct dcl_ctx {
   uint8_t *cmt = nullptr, *cmt_init = nullptr;    // committed flags [B][T] (Eq. threshold_pd decoding)
   int* derr = nullptr;
   float *rope_cos = nullptr, *rope_sin = nullptr;
+  float2* rope_cs = nullptr;  // the same as {cos, sin} pairs, position-major (few-row GEMMs)
   float* snap = nullptr;  // residual stream after the embedding and after each layer (debug)
   int* gemm_flags = nullptr;  // split-K counters of the step's GEMMs (zero between launches)
   size_t gemm_flags_n = 0;
@@ -89,11 +96,13 @@ struct dcl_ctx {
   std::vector<GemmPlan> plans;  // 4 per layer + LM head
   std::vector<AttnPlan> attn_plans;  // one per layer
   bool kv_fused = false;  // the QKV GEMMs write k and v^T (no transpose launch)
+  // few-row GEMMs of the layers (qkv, o, gate/up, down; 4 per layer): [0] for up to 32 rows,
+  // [1] for up to FEW_MAX_ROWS; empty where no step of this shape takes them
+  std::vector<FewPlan> few[2];
   cudaGraphExec_t gexec = nullptr;
   bool profiling = false;
-  std::vector<Launch> launches;
-  size_t launch_i = 0;
-  bool profiled_step = false;
+  ProfGraph prof[STEP_BRANCHES];  // profiling: one graph per branch, the host takes the step's
+  int prof_last = -1;             // the branch of the last profiled step
   int32_t* h_done = nullptr;  // pinned [2]
   cudaEvent_t ev_done[2] = {nullptr, nullptr};
 };
@@ -184,18 +193,18 @@ dcl_status check_device(dcl_ctx* c) {
 // ------------------------------------------------------------------ the step
 struct Enq {
   dcl_ctx* c;
-  bool prof;
+  ProfGraph* prof;  // timing events go here, or NULL
   cudaError_t err = cudaSuccess;
   const char* what = nullptr;
   void begin(int kind) {
     if (!prof || err != cudaSuccess) return;
-    if (c->launch_i >= c->launches.size()) {
+    if (prof->n >= prof->launches.size()) {
       Launch l{kind, nullptr, nullptr};
       cudaEventCreate(&l.start);
       cudaEventCreate(&l.stop);
-      c->launches.push_back(l);
+      prof->launches.push_back(l);
     }
-    Launch& l = c->launches[c->launch_i];
+    Launch& l = prof->launches[prof->n];
     l.kind = kind;
     err = cudaEventRecordWithFlags(l.start, c->stream, cudaEventRecordExternal);
   }
@@ -205,25 +214,30 @@ struct Enq {
       what = name;
     }
     if (!prof || err != cudaSuccess) return;
-    err = cudaEventRecordWithFlags(c->launches[c->launch_i].stop, c->stream, cudaEventRecordExternal);
-    ++c->launch_i;
+    err = cudaEventRecordWithFlags(prof->launches[prof->n].stop, c->stream, cudaEventRecordExternal);
+    ++prof->n;
   }
 };
 
-// Enqueue the forward (and, if with_dcv, the acceptance) on the context stream.  With
-// h_in the forward starts at block first_layer from that residual stream (row b*T + t;
-// no re-mask, no embedding; full recompute only).
-cudaError_t enqueue_step(dcl_ctx* c, bool with_dcv, bool prof, bool snapshots, const char** what,
-                         int first_layer = 0, const float* h_in = nullptr) {
+// The step's first launch: the rows it computes (and, inside a step graph with branches, the
+// choice among them).
+void enqueue_rows(dcl_ctx* c, Enq& q, bool update, cudaGraphConditionalHandle select) {
+  q.begin(DCL_K_ROWPLAN);
+  q.end(row_plan_launch(c->rp, c->p, c->B, c->N, c->T, c->dcfg.block_len, c->dcfg.kv_cache, update ? 1 : 0, c->x,
+                        c->dcfg.acceptance ? 0 : c->window, c->cfg.mask_id, select, c->stream),
+        "row_plan");
+}
+
+// Enqueue the forward (and, if with_dcv, the acceptance) on the context stream, with the GEMMs
+// of the given branch.  With h_in the forward starts at block first_layer from that residual
+// stream (row b*T + t; no re-mask, no embedding; full recompute only).
+void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapshots, int first_layer = 0,
+                     const float* h_in = nullptr) {
   const dcl_model_config& m = c->cfg;
   const int R = c->B * c->T;
   const int d = m.d_model;
-  Enq q{c, prof};
-  if (prof) c->launch_i = 0;
-  q.begin(DCL_K_ROWPLAN);
-  q.end(row_plan_launch(c->rp, c->p, c->B, c->N, c->T, c->dcfg.block_len, c->dcfg.kv_cache, with_dcv ? 1 : 0,
-                        c->x, c->dcfg.acceptance ? 0 : c->window, m.mask_id, c->stream),
-        "row_plan");
+  const std::vector<FewPlan>* few = branch == STEP_PAIR ? nullptr : &c->few[branch == STEP_FEW32 ? 0 : 1];
+  const int rows = std::min(R, branch == STEP_FEW32 ? 32 : branch == STEP_FEW ? FEW_MAX_ROWS : R);  // at most
   if (h_in) {
     if (q.err == cudaSuccess)
       q.err = cudaMemcpyAsync(c->h, h_in, sizeof(float) * R * d, cudaMemcpyDeviceToDevice, c->stream);
@@ -241,10 +255,12 @@ cudaError_t enqueue_step(dcl_ctx* c, bool with_dcv, bool prof, bool snapshots, c
   for (int l = first_layer; l < m.n_layers && q.err == cudaSuccess; ++l) {
     const Layer& L = c->layers[l];
     const GemmPlan* P = &c->plans[4 * l];
+    const FewPlan* F = few ? &(*few)[4 * l] : nullptr;
     q.begin(DCL_K_RMSNORM);
-    q.end(rmsnorm_launch(c->h, L.attn_norm, c->xn, R, d, m.rms_eps, c->rp.counts, nullptr, c->stream), "rmsnorm");
+    q.end(rmsnorm_launch(c->h, L.attn_norm, c->xn, rows, d, m.rms_eps, c->rp.counts, nullptr, F != nullptr, c->stream),
+          "rmsnorm");
     q.begin(DCL_K_GEMM_QKV);
-    q.end(gemm_launch(P[0], c->derr, c->stream), "gemm_qkv");
+    q.end(F ? few_launch(F[0], c->derr, c->stream) : gemm_launch(P[0], c->derr, c->stream), "gemm_qkv");
     if (!c->kv_fused) {
       q.begin(DCL_K_VTRANSPOSE);
       q.end(attention_transpose_launch(c->attn_plans[l], c->stream), "v_transpose");
@@ -252,17 +268,18 @@ cudaError_t enqueue_step(dcl_ctx* c, bool with_dcv, bool prof, bool snapshots, c
     q.begin(DCL_K_ATTENTION);
     q.end(attention_core_launch(c->attn_plans[l], c->derr, c->stream), "attention");
     q.begin(DCL_K_GEMM_O);
-    q.end(gemm_launch(P[1], c->derr, c->stream), "gemm_o");
+    q.end(F ? few_launch(F[1], c->derr, c->stream) : gemm_launch(P[1], c->derr, c->stream), "gemm_o");
     q.begin(DCL_K_RMSNORM);
-    q.end(rmsnorm_launch(c->h, L.mlp_norm, c->xn, R, d, m.rms_eps, c->rp.counts, nullptr, c->stream), "rmsnorm");
-    if (P[2].fuse) {  // gate/up + SwiGLU and down + residual in one launch
+    q.end(rmsnorm_launch(c->h, L.mlp_norm, c->xn, rows, d, m.rms_eps, c->rp.counts, nullptr, F != nullptr, c->stream),
+          "rmsnorm");
+    if (!F && P[2].fuse) {  // gate/up + SwiGLU and down + residual in one launch
       q.begin(DCL_K_GEMM_MLP);
       q.end(gemm_launch(P[2], c->derr, c->stream), "gemm_mlp");
     } else {
       q.begin(DCL_K_GEMM_GATEUP);
-      q.end(gemm_launch(P[2], c->derr, c->stream), "gemm_gateup");
+      q.end(F ? few_launch(F[2], c->derr, c->stream) : gemm_launch(P[2], c->derr, c->stream), "gemm_gateup");
       q.begin(DCL_K_GEMM_DOWN);
-      q.end(gemm_launch(P[3], c->derr, c->stream), "gemm_down");
+      q.end(F ? few_launch(F[3], c->derr, c->stream) : gemm_launch(P[3], c->derr, c->stream), "gemm_down");
     }
     if (snapshots && q.err == cudaSuccess)
       q.err = cudaMemcpyAsync(c->snap + (size_t)(l + 1) * R * d, c->h, sizeof(float) * R * d,
@@ -271,7 +288,7 @@ cudaError_t enqueue_step(dcl_ctx* c, bool with_dcv, bool prof, bool snapshots, c
   // final norm on the computed generation rows only (LM row j <- computed row lm_src[j])
   q.begin(DCL_K_RMSNORM);
   q.end(rmsnorm_launch(c->h, c->final_norm, c->xg, c->B * c->M, d, m.rms_eps, c->rp.counts + 1, c->rp.lm_src,
-                       c->stream),
+                       false, c->stream),
         "final_rmsnorm");
   q.begin(DCL_K_GEMM_LMHEAD);
   q.end(gemm_launch(c->plans[4 * m.n_layers], c->derr, c->stream), "gemm_lmhead");
@@ -294,28 +311,129 @@ cudaError_t enqueue_step(dcl_ctx* c, bool with_dcv, bool prof, bool snapshots, c
                             c->done_count, c->cmt, c->rp.kcap, c->stream),
           "dcv_commit");
   }
-  if (what) *what = q.what;
-  return q.err;
+}
+
+// The branch of the next step: by its rows, as the row plan counts them.  Fixed by the shape
+// without a key / value cache; else read from the device (synchronises).
+dcl_status current_branch(dcl_ctx* c, int* out) {
+  *out = STEP_PAIR;
+  if (c->few[0].empty()) return DCL_OK;
+  if (!c->dcfg.kv_cache) {
+    *out = step_branch(c->B * c->T);
+    return DCL_OK;
+  }
+  std::vector<int32_t> ph(c->B), pe(c->B);
+  CUDA_TRY(c, cudaMemcpyAsync(ph.data(), c->p, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(pe.data(), c->rp.pe_cache, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  const int Bk = c->dcfg.block_len;
+  long rows = 0;
+  for (int b = 0; b < c->B; ++b) {
+    if (ph[b] >= c->T) continue;
+    const int end = c->N + Bk * ((ph[b] - c->N) / Bk);
+    const bool fresh = pe[b] == end;
+    const int start = fresh ? end : 0;
+    rows += (c->dcfg.kv_cache == 2 && start != 0 ? std::min(end + Bk, c->T) : c->T) - start;
+  }
+  *out = step_branch((int)rows);
+  return DCL_OK;
+}
+
+void destroy_graphs(dcl_ctx* c) {
+  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  c->gexec = nullptr;
+  for (ProfGraph& g : c->prof) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    g.exec = nullptr;
+  }
+  c->prof_last = -1;
+}
+
+// Capture onto the context stream, into g, what body(Enq&) enqueues.
+template <typename Body>
+dcl_status capture_into(dcl_ctx* c, cudaGraph_t g, ProfGraph* prof, Body body) {
+  CUDA_TRY(c, cudaStreamBeginCaptureToGraph(c->stream, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  Enq q{c, prof};
+  body(q);
+  cudaGraph_t same = nullptr;
+  const cudaError_t e2 = cudaStreamEndCapture(c->stream, &same);
+  if (q.err != cudaSuccess)
+    return fail(c, DCL_ERR_CUDA, "capturing the step failed at %s: %s", q.what ? q.what : "?",
+                cudaGetErrorString(q.err));
+  if (e2 != cudaSuccess) return fail(c, DCL_ERR_CUDA, "end capture: %s", cudaGetErrorString(e2));
+  return DCL_OK;
+}
+
+// The step whose GEMMs follow its row count: the row plan, then a switch node whose bodies are
+// the rest of the step with each branch's GEMMs (the row plan sets the switch on the device, so
+// a step stays one graph launch without a host round trip).
+dcl_status capture_switch(dcl_ctx* c, cudaGraph_t g) {
+  cudaGraphConditionalHandle select = 0;
+  CUDA_TRY(c, cudaGraphConditionalHandleCreate(&select, g, STEP_PAIR, cudaGraphCondAssignDefault));
+  dcl_status s = capture_into(c, g, nullptr, [&](Enq& q) { enqueue_rows(c, q, true, select); });
+  if (s != DCL_OK) return s;
+  cudaGraphNode_t rows = nullptr, node = nullptr;
+  size_t n = 1;
+  CUDA_TRY(c, cudaGraphGetNodes(g, &rows, &n));
+  cudaGraphNodeParams prm = {};
+  prm.type = cudaGraphNodeTypeConditional;
+  prm.conditional.handle = select;
+  prm.conditional.type = cudaGraphCondTypeSwitch;
+  prm.conditional.size = STEP_BRANCHES;
+  CUDA_TRY(c, cudaGraphAddNode(&node, g, &rows, nullptr, 1, &prm));
+  for (int br = 0; br < STEP_BRANCHES && s == DCL_OK; ++br)
+    s = capture_into(c, prm.conditional.phGraph_out[br], nullptr,
+                     [&](Enq& q) { enqueue_forward(c, q, br, true, false); });
+  return s;
+}
+
+dcl_status build_exec(dcl_ctx* c, cudaGraphExec_t* exec, bool with_switch, int branch, ProfGraph* prof) {
+  cudaGraph_t g = nullptr;
+  CUDA_TRY(c, cudaGraphCreate(&g, 0));
+  if (prof) prof->n = 0;
+  dcl_status s = with_switch ? capture_switch(c, g) : capture_into(c, g, prof, [&](Enq& q) {
+    enqueue_rows(c, q, true, 0);
+    enqueue_forward(c, q, branch, true, false);
+  });
+  if (s == DCL_OK) {
+    const cudaError_t e = cudaGraphInstantiate(exec, g, 0);
+    if (e != cudaSuccess) s = fail(c, DCL_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
+  }
+  cudaGraphDestroy(g);
+  return s;
 }
 
 dcl_status build_graph(dcl_ctx* c) {
-  if (c->gexec) {
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
+  destroy_graphs(c);
+  const bool by_rows = !c->few[0].empty() && c->dcfg.kv_cache;
+  const int fixed = c->few[0].empty() ? (int)STEP_PAIR : step_branch(c->B * c->T);
+  if (!c->profiling) return build_exec(c, &c->gexec, by_rows, fixed, nullptr);
+  for (int br = 0; br < STEP_BRANCHES; ++br)
+    if (by_rows || br == fixed) {
+      const dcl_status s = build_exec(c, &c->prof[br].exec, false, br, &c->prof[br]);
+      if (s != DCL_OK) return s;
+    }
+  return DCL_OK;
+}
+
+bool have_graph(const dcl_ctx* c) {
+  if (c->gexec) return true;
+  for (const ProfGraph& g : c->prof)
+    if (g.exec) return true;
+  return false;
+}
+
+// One step on the context stream.
+dcl_status launch_step(dcl_ctx* c) {
+  if (!c->profiling) {
+    CUDA_TRY(c, cudaGraphLaunch(c->gexec, c->stream));
+    return DCL_OK;
   }
-  cudaGraph_t g = nullptr;
-  CUDA_TRY(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  const char* what = nullptr;
-  cudaError_t e = enqueue_step(c, true, c->profiling, false, &what);
-  cudaError_t e2 = cudaStreamEndCapture(c->stream, &g);
-  if (e != cudaSuccess)
-    return fail(c, DCL_ERR_CUDA, "capturing the step failed at %s: %s", what ? what : "?",
-                cudaGetErrorString(e));
-  if (e2 != cudaSuccess) return fail(c, DCL_ERR_CUDA, "end capture: %s", cudaGetErrorString(e2));
-  e = cudaGraphInstantiate(&c->gexec, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
-  c->profiled_step = false;
+  int br;
+  const dcl_status s = current_branch(c, &br);
+  if (s != DCL_OK) return s;
+  CUDA_TRY(c, cudaGraphLaunch(c->prof[br].exec, c->stream));
+  c->prof_last = br;
   return DCL_OK;
 }
 
@@ -445,6 +563,54 @@ dcl_status build_plans(dcl_ctx* c) {
     return fail(c, DCL_ERR_UNSUPPORTED, "LM-head plan: %s", why ? why : "?");
   if (c->plans[4 * m.n_layers].streamk)
     return fail(c, DCL_ERR_UNSUPPORTED, "stream-K needs a fixed row count; the step's GEMMs cannot use it");
+  // the few-row GEMMs, where a step of this shape can have so few rows (a tile override keeps
+  // every step on the GEMMs it names)
+  c->few[0].clear();
+  c->few[1].clear();
+  const bool planned = t_qkv == kTilePair && t_o == kTilePair && t_gu == kTilePair && t_down == kTilePair;
+  if (planned && (cached || R <= FEW_MAX_ROWS)) {
+    bool ok = true;
+    for (int v = 0; v < 2 && ok; ++v) {
+      const int nt = v == 0 ? 32 : FEW_MAX_ROWS;
+      c->few[v].assign(4 * m.n_layers, FewPlan{});
+      for (int l = 0; l < m.n_layers && ok; ++l) {
+        const Layer& L = c->layers[l];
+        FewPlan* F = &c->few[v][4 * l];
+        FewEpi base;
+        base.m_dev = c->rp.counts;
+        base.w_early = 1;
+        FewEpi fq = base;
+        fq.out = c->qkv;
+        fq.ldo = nqkv;
+        fq.rope = c->rope_cs;
+        fq.rope_cols = (H + G) * hd;
+        fq.head_dim = hd;
+        fq.row_pos = c->rp.row_pos;
+        fq.row_seq = c->rp.row_seq;
+        if (c->kv_fused) {
+          fq.k_col0 = H * hd;
+          fq.kdst = kbuf_of(l);
+          fq.vdst = vbuf_of(l);
+          fq.G = G;
+          fq.T = c->T;
+          fq.Tp = Tp;
+        }
+        FewEpi fh = base, fa = base;
+        fh.out = c->h;
+        fh.ldo = d;
+        fa.out = c->act;
+        fa.ldo = m.ffn_dim;
+        ok = few_plan(&F[0], c->xn, R, d, L.wqkv, nqkv, EPI_QKV_ROPE, fq, c->num_sms, nt) == cudaSuccess &&
+             few_plan(&F[1], c->attn, R, H * hd, L.wo, d, EPI_RESID_F32, fh, c->num_sms, nt) == cudaSuccess &&
+             few_plan(&F[2], c->xn, R, d, L.wgu, 2 * m.ffn_dim, EPI_SWIGLU, fa, c->num_sms, nt) == cudaSuccess &&
+             few_plan(&F[3], c->act, R, m.ffn_dim, L.wdown, d, EPI_RESID_F32, fh, c->num_sms, nt) == cudaSuccess;
+      }
+    }
+    if (!ok) {  // (a shape only the pair GEMMs take)
+      c->few[0].clear();
+      c->few[1].clear();
+    }
+  }
   // split-K counters and partials, shared by the step's GEMMs (they run one after another)
   size_t need_f = 0, need_w = 0;
   for (const GemmPlan& p : c->plans) {
@@ -453,10 +619,7 @@ dcl_status build_plans(dcl_ctx* c) {
   }
   if (need_f > c->gemm_flags_n || need_w > c->gemm_ws_n) {
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // no launch may still use the old buffers
-    if (c->gexec) {
-      cudaGraphExecDestroy(c->gexec);
-      c->gexec = nullptr;
-    }
+    destroy_graphs(c);
   }
   if (need_f > c->gemm_flags_n) {
     dev_free_one(c, c->gemm_flags);
@@ -684,10 +847,11 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
     c->cmt_init = (uint8_t*)dev_alloc(c, R);
     c->rope_cos = (float*)dev_alloc(c, 4 * (size_t)max_seq * hd / 2);
     c->rope_sin = (float*)dev_alloc(c, 4 * (size_t)max_seq * hd / 2);
+    c->rope_cs = (float2*)dev_alloc(c, 8 * (size_t)max_seq * hd / 2);
     if (!c->wbuf || !c->h || !c->xn || !c->qkv || !c->attn || !c->vt || !c->kbuf || !c->rp_buf || !c->act || !c->xg || !c->part || !c->ent_part ||
         !c->ent || !c->conf || !c->jpde || !c->top1 ||
         !c->p1 || !c->p2 || !c->x || !c->p || !c->k || !c->steps || !c->done_count || !c->x_init || !c->p_init || !c->cmt || !c->cmt_init || !c->rope_cos ||
-        !c->rope_sin) {
+        !c->rope_sin || !c->rope_cs) {
       dev_free_all(c);
       release_stream(c);
       delete c;
@@ -712,7 +876,7 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
     c->rp.seq_len = c->rp.seq_off + max_batch;
     c->rp.pe_cache = c->rp.seq_len + max_batch;
     c->rp.kcap = c->rp.pe_cache + max_batch;
-    if (rope_table_build(c->rope_cos, c->rope_sin, max_seq, (int)hd, m.rope_theta, c->stream) != cudaSuccess) {
+    if (rope_table_build(c->rope_cos, c->rope_sin, c->rope_cs, max_seq, (int)hd, m.rope_theta, c->stream) != cudaSuccess) {
       dev_free_all(c);
       release_stream(c);
       delete c;
@@ -734,11 +898,12 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
 void dcl_destroy(dcl_ctx* c) {
   if (!c) return;
   if (c->stream) cudaStreamSynchronize(c->stream);
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
-  for (auto& l : c->launches) {
-    cudaEventDestroy(l.start);
-    cudaEventDestroy(l.stop);
-  }
+  destroy_graphs(c);
+  for (ProfGraph& g : c->prof)
+    for (Launch& l : g.launches) {
+      cudaEventDestroy(l.start);
+      cudaEventDestroy(l.stop);
+    }
   if (c->ev_done[0]) cudaEventDestroy(c->ev_done[0]);
   if (c->ev_done[1]) cudaEventDestroy(c->ev_done[1]);
   if (c->h_done) cudaFreeHost(c->h_done);
@@ -844,7 +1009,7 @@ dcl_status dcl_set_prompt(dcl_ctx* c, int32_t batch, const int32_t* prompt, int3
     s = build_plans(c);
     if (s != DCL_OK) return s;
   }
-  if (reshape || redcv || !c->gexec) {
+  if (reshape || redcv || !have_graph(c)) {
     s = build_graph(c);
     if (s != DCL_OK) return s;
   }
@@ -855,8 +1020,8 @@ dcl_status dcl_set_prompt(dcl_ctx* c, int32_t batch, const int32_t* prompt, int3
 dcl_status dcl_step(dcl_ctx* c, int32_t* k_out) {
   if (!c) return DCL_ERR_INVALID_ARG;
   if (!c->prompt_set) return fail(c, DCL_ERR_STATE, "dcl_step before dcl_set_prompt");
-  CUDA_TRY(c, cudaGraphLaunch(c->gexec, c->stream));
-  c->profiled_step = c->profiling;
+  const dcl_status s = launch_step(c);
+  if (s != DCL_OK) return s;
   if (k_out) {
     CUDA_TRY(c, cudaMemcpyAsync(k_out, c->k, 4 * c->B, cudaMemcpyDeviceToHost, c->stream));
     return check_device(c);
@@ -876,7 +1041,8 @@ dcl_status dcl_generate(dcl_ctx* c, int32_t max_steps, int32_t* out, dcl_stats* 
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   done = c->h_done[0] >= c->B;
   while (!done && launched < max_steps) {
-    CUDA_TRY(c, cudaGraphLaunch(c->gexec, c->stream));
+    const dcl_status ls = launch_step(c);
+    if (ls != DCL_OK) return ls;
     const int slot = launched & 1;
     CUDA_TRY(c, cudaMemcpyAsync(&c->h_done[slot], c->done_count, 4, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaEventRecord(c->ev_done[slot], c->stream));
@@ -888,7 +1054,6 @@ dcl_status dcl_generate(dcl_ctx* c, int32_t max_steps, int32_t* out, dcl_stats* 
   }
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   if (launched > 0 && c->h_done[(launched - 1) & 1] >= c->B) done = true;
-  c->profiled_step = c->profiling && launched > 0;
   dcl_status s = check_device(c);
   if (s != DCL_OK) return s;
   std::vector<int32_t> ph(c->B), sh(c->B);
@@ -977,9 +1142,14 @@ dcl_status forward_debug_impl(dcl_ctx* c, int layer, const float* h_in, bool com
     if (!c->snap) return fail(c, DCL_ERR_OOM, "snapshot buffer allocation failed");
     c->snap_rows = R;
   }
-  const char* what = nullptr;
-  cudaError_t e = enqueue_step(c, commit, false, true, &what, layer, h_in);
-  if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "forward failed at %s: %s", what ? what : "?", cudaGetErrorString(e));
+  int br;  // (the predictions are those of the step itself: the same GEMMs)
+  const dcl_status bs = current_branch(c, &br);
+  if (bs != DCL_OK) return bs;
+  Enq q{c, nullptr};
+  enqueue_rows(c, q, commit, 0);
+  enqueue_forward(c, q, br, commit, true, layer, h_in);
+  if (q.err != cudaSuccess)
+    return fail(c, DCL_ERR_CUDA, "forward failed at %s: %s", q.what ? q.what : "?", cudaGetErrorString(q.err));
   const size_t G = (size_t)c->B * c->M;
   if (top1_dev) CUDA_TRY(c, cudaMemcpyAsync(top1_dev, c->top1, 4 * G, cudaMemcpyDeviceToDevice, c->stream));
   if (p1_dev) CUDA_TRY(c, cudaMemcpyAsync(p1_dev, c->p1, 4 * G, cudaMemcpyDeviceToDevice, c->stream));
@@ -1079,7 +1249,7 @@ dcl_status dcl_op_rmsnorm(dcl_ctx* c, const float* x_dev, const void* gain_dev, 
   if (!c) return DCL_ERR_INVALID_ARG;
   if (!x_dev || !gain_dev || !y_dev || rows <= 0 || d <= 0 || d % 4) return fail(c, DCL_ERR_INVALID_ARG, "bad rmsnorm args");
   CUDA_TRY(c, rmsnorm_launch(x_dev, static_cast<const __nv_bfloat16*>(gain_dev), static_cast<__nv_bfloat16*>(y_dev),
-                             rows, d, eps, nullptr, nullptr, c->stream));
+                             rows, d, eps, nullptr, nullptr, false, c->stream));
   return DCL_OK;
 }
 
@@ -1096,6 +1266,18 @@ dcl_status dcl_op_linear(dcl_ctx* c, const void* a_dev, const void* w_dev, void*
   const char* why = nullptr;
   if (gemm_plan(&pl, a_dev, M, K, w_dev, N, mode == 0 ? EPI_BF16 : EPI_RESID_F32, ep, c->num_sms, tile, &why))
     return fail(c, DCL_ERR_INVALID_ARG, "%s", why ? why : "bad GEMM shape");
+  if (tile == 0 && M <= FEW_MAX_ROWS) {  // as the step's GEMMs of so few rows
+    FewPlan fp;
+    FewEpi fe;
+    fe.out = out_dev;
+    fe.ldo = N;
+    if (few_plan(&fp, a_dev, M, K, w_dev, N, mode == 0 ? EPI_BF16 : EPI_RESID_F32, fe, c->num_sms,
+                 M <= 32 ? 32 : FEW_MAX_ROWS) == cudaSuccess) {
+      const cudaError_t e = few_launch(fp, c->derr, c->stream);
+      if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "GEMM launch: %s", cudaGetErrorString(e));
+      return check_device(c);
+    }
+  }
   dcl_status s = attach_scratch(c, &pl);
   if (s != DCL_OK) return s;
   const cudaError_t e = gemm_launch(pl, c->derr, c->stream);
@@ -1253,15 +1435,16 @@ dcl_status dcl_set_profiling(dcl_ctx* c, int32_t enable) {
 
 dcl_status dcl_profile_last_step(dcl_ctx* c, float* ms, int32_t* kind, int32_t cap, int32_t* n) {
   if (!c) return DCL_ERR_INVALID_ARG;
-  if (!c->profiling || !c->profiled_step) return fail(c, DCL_ERR_STATE, "no profiled step has run");
+  if (!c->profiling || c->prof_last < 0) return fail(c, DCL_ERR_STATE, "no profiled step has run");
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  const int cnt = (int)c->launch_i;
+  const std::vector<Launch>& ls = c->prof[c->prof_last].launches;
+  const int cnt = (int)c->prof[c->prof_last].n;
   int w = 0;
   for (int i = 0; i < cnt && w < cap; ++i, ++w) {
     float t = 0.f;
-    CUDA_TRY(c, cudaEventElapsedTime(&t, c->launches[i].start, c->launches[i].stop));
+    CUDA_TRY(c, cudaEventElapsedTime(&t, ls[i].start, ls[i].stop));
     if (ms) ms[w] = t;
-    if (kind) kind[w] = c->launches[i].kind;
+    if (kind) kind[w] = ls[i].kind;
   }
   if (n) *n = w;
   return DCL_OK;

@@ -1,0 +1,481 @@
+// GEMMs of a step with few rows (at most FEW_MAX_ROWS tokens: the current block or a short
+// suffix under the key / value caches, small full recomputes):
+//   out = X[rows][K] @ W[N][K]^T   with the step's epilogues fused.
+//
+// What bounds them is the weight stream: every weight is read once for a handful of tokens.
+// The CTA-pair kernel puts tokens on the MMA's 256-row side, so that 32 live rows cost the
+// MMA time of 256 (18 us per 256 x 256 x 4096 tile) on as many SM pairs as there are column
+// tiles (48 of 76 for QKV, 16 for O).  Here the operands are swapped: 128 weight rows on the
+// M side, the tokens (rounded up to 32) on the N side, so the MMA time follows the tokens, and
+// each tile of 128 weight rows is split by K over a cluster of S CTAs.  S is the largest power
+// of two up to 8 that leaves a CTA a K block and the grid within two CTAs per SM.
+//
+// One CTA = one tile's share of K (192 threads: TMA producer, MMA issuer, four epilogue
+// warps).  Its fp32 sum goes from TMEM to its idle operand ring; after a cluster barrier each
+// CTA of the cluster finishes nt / S tokens, adding the S sums through distributed shared
+// memory in K order (bit-reproducible), so the tail is a barrier and one short pass (about 2.5
+// us) instead of a round trip of partial sums through L2 (which made these launches no faster
+// than the pair kernel's).
+//
+// A CTA takes less than half of an SM's shared memory, TMEM and registers, so that under
+// programmatic dependent launch the next GEMM of the step is resident beside the running one
+// and fills its ring with weights, which depend on no earlier kernel, before its
+// dependent-launch wait: the HBM keeps streaming across kernel boundaries.  More CTAs (more
+// bytes in flight) stream faster: 192 CTAs of the gate/up GEMM read 201 MB in 29 us (6.9
+// TB/s), 96 CTAs of an unsplit QKV 100 MB in 22 us, 192 in 16 us.
+//
+// Measured per step, 8 layers of the LLaDA-8B shape at T = 1536: 32 rows 1415 -> 1092 us, 96
+// rows 1430 -> 1208 us; the 2-layer test model (96 rows, latency) 119 -> 81 us.
+#include <string.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "tc_ptx.cuh"
+
+namespace dcl {
+namespace {
+
+constexpr int FW_THREADS = 192;
+constexpr int FW_BK = 64;                 // K block: one 128-byte swizzle row of bf16
+constexpr int FW_TILE = 128;              // weight rows of a tile
+constexpr int FW_W_BYTES = FW_TILE * 128; // a K block of them
+constexpr int FW_XBOX_BYTES = 32 * 128;   // 32 tokens x one K block
+constexpr int FW_MAX_STAGES = 5;
+constexpr int FW_BARS = 256 + 2 * 4 * FEW_MAX_ROWS;  // barriers, then the tokens' positions and sequences
+constexpr size_t FW_SMEM = 112 * 1024;
+constexpr int FW_RING = (int)FW_SMEM - 1024 - FW_BARS;
+constexpr int FW_PITCH = FW_TILE + 4;     // fp32 per token of a staged sum
+static_assert(FEW_MAX_ROWS * FW_PITCH * 4 <= FW_RING, "the staged sum lives in the operand ring");
+static_assert(8 * (2 * FW_MAX_STAGES + 1) + 16 <= 256, "barrier area");
+
+struct FewArgs {
+  int nkb;     // K blocks
+  int nt_max;  // tokens the launch may hold (32 or FEW_MAX_ROWS)
+  int N, M;
+  FewEpi ep;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// (orders nothing: the arrive does not wait for this thread's global stores)
+__device__ __forceinline__ void cluster_sync_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_cluster(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr));
+  return v;
+}
+// h += v without a return value (one add per element: no order to depend on)
+__device__ __forceinline__ void red_add_v4(float* p, const float4& v) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+// Four consecutive rows' sums (address `at` in every CTA of the cluster) of NP tokens, `step`
+// bytes apart, added in K order.  All S * NP loads are issued before any is used, 16 bytes
+// each: distributed shared memory is slow per access (adding rank after rank, 4 bytes a
+// load, the pass took 5 us).
+template <int S, int NP>
+__device__ __forceinline__ void cluster_sums(uint32_t at, uint32_t step, int n, float4 (&x)[NP]) {
+  float4 v[S][NP];
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    const uint32_t from = S == 1 ? at : map_cluster(at, s);
+#pragma unroll
+    for (int i = 0; i < NP; ++i)
+      if (i < n) v[s][i] = S == 1 ? ld_shared_v4(from + i * step) : ld_cluster_v4(from + i * step);
+  }
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    x[i] = v[0][i];
+#pragma unroll
+    for (int s = 1; s < S; ++s) {
+      x[i].x += v[s][i].x;
+      x[i].y += v[s][i].y;
+      x[i].z += v[s][i].z;
+      x[i].w += v[s][i].w;
+    }
+  }
+}
+
+__device__ __forceinline__ void store_bf16x4(__nv_bfloat16* o, float a, float b, float c, float d) {
+  *reinterpret_cast<uint2*>(o) = make_uint2(pack_bf16x2(a, b), pack_bf16x2(c, d));
+}
+
+// Tokens t0 .. t1 - 1 of the tile, by the 128 epilogue threads (et), four consecutive rows per
+// thread.  sum: the staged sums [token][FW_PITCH], at the same shared address in each of the
+// cluster's S CTAs.
+template <int EPI, int S>
+__device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u, int t0, int t1, int et,
+                                           const int* pos_s, const int* seq_s) {
+  const FewEpi& ep = a.ep;
+  const int n0 = u * FW_TILE;
+  constexpr int NP = S >= 4 ? 2 : 4;  // tokens in flight per thread
+  constexpr uint32_t TOK = FW_PITCH * 4;
+  auto at = [&](int t, int r) { return sum + (uint32_t)t * TOK + (uint32_t)(4 * r); };
+  if constexpr (EPI == EPI_BF16 || EPI == EPI_RESID_F32) {  // a warp per token
+    const int r = 4 * (et & 31), n = n0 + r;
+    if (n >= a.N) return;
+#pragma unroll 1
+    for (int t = t0 + (et >> 5); t < t1; t += 4 * NP) {
+      float4 x[NP];
+      const int m = (t1 - t + 3) >> 2;
+      cluster_sums<S, NP>(at(t, r), 4 * TOK, m, x);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        if (i >= m) continue;
+        const size_t o = (size_t)(t + 4 * i) * ep.ldo + n;
+        if constexpr (EPI == EPI_BF16)
+          store_bf16x4(static_cast<__nv_bfloat16*>(ep.out) + o, x[i].x, x[i].y, x[i].z, x[i].w);
+        else
+          red_add_v4(static_cast<float*>(ep.out) + o, x[i]);
+      }
+    }
+  } else if constexpr (EPI == EPI_SWIGLU) {  // gate rows j .. j + 3 and up rows 64 + j ..; half a warp per token
+    const int j = 4 * (et & 15);
+#pragma unroll 1
+    for (int t = t0 + (et >> 4); t < t1; t += 8 * NP) {
+      float4 g[NP], v[NP];
+      const int m = (t1 - t + 7) >> 3;
+      cluster_sums<S, NP>(at(t, j), 8 * TOK, m, g);
+      cluster_sums<S, NP>(at(t, 64 + j), 8 * TOK, m, v);
+      auto act = [](float x, float y) { return __fdividef(x, 1.0f + __expf(-x)) * y; };
+#pragma unroll
+      for (int i = 0; i < NP; ++i)
+        if (i < m)
+          store_bf16x4(static_cast<__nv_bfloat16*>(ep.out) + (size_t)(t + 8 * i) * ep.ldo + u * 64 + j,
+                       act(g[i].x, v[i].x), act(g[i].y, v[i].y), act(g[i].z, v[i].z), act(g[i].w, v[i].w));
+    }
+  } else if (n0 >= ep.rope_cols && ep.vdst) {
+    // v leaves transposed, in fp16 holding the bf16 values: four channels x four tokens per
+    // thread, positions contiguous.  (Groups of 32 rows are consecutive positions of one
+    // sequence from a multiple of 32, and a CTA's tokens a multiple of 4: 8-byte stores.)
+    const int r = 4 * (et & 31);
+    if (n0 + r >= a.N) return;
+#pragma unroll 1
+    for (int t = t0 + 4 * (et >> 5); t < t1; t += 16) {
+      float4 x[4];
+      cluster_sums<S, 4>(at(t, r), TOK, 4, x);
+      auto h = [](float f) { return __bfloat162float(__float2bfloat16_rn(f)); };
+      __half* o = ep.vdst + ((size_t)seq_s[t] * ep.G * ep.head_dim + (n0 + r - ep.rope_cols)) * ep.Tp + pos_s[t];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        auto f = [&](int i) { return h(c == 0 ? x[i].x : c == 1 ? x[i].y : c == 2 ? x[i].z : x[i].w); };
+        *reinterpret_cast<uint2*>(o + (size_t)c * ep.Tp) = make_uint2(pack_f16x2(f(0), f(1)), pack_f16x2(f(2), f(3)));
+      }
+    }
+  } else {  // q, k (and v without a store of its own): components j .. j + 3 and j + head_dim / 2 .. of a head
+    const int half = ep.head_dim >> 1, jj = 4 * (et & 15), j = jj & (half - 1);
+    const int r0 = jj + (jj & ~(half - 1)), r1 = r0 + half;
+    if (n0 + r1 >= a.N) return;
+    const bool rope = n0 < ep.rope_cols, to_k = rope && ep.kdst && n0 >= ep.k_col0;
+    constexpr int NQ = S >= 4 ? 1 : 2;
+#pragma unroll 1
+    for (int t = t0 + (et >> 4); t < t1; t += 8 * NQ) {
+      float4 x[NQ], y[NQ], c[NQ], d[NQ];  // c: {cos, sin} of j, j + 1; d: of j + 2, j + 3
+      const int m = (t1 - t + 7) >> 3;
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        c[i] = d[i] = make_float4(1.f, 0.f, 1.f, 0.f);
+        if (rope && i < m) {
+          const float4* cs = reinterpret_cast<const float4*>(ep.rope + (size_t)pos_s[t + 8 * i] * half + j);
+          c[i] = __ldg(cs);
+          d[i] = __ldg(cs + 1);
+        }
+      }
+      cluster_sums<S, NQ>(at(t, r0), 8 * TOK, m, x);
+      cluster_sums<S, NQ>(at(t, r1), 8 * TOK, m, y);
+#pragma unroll
+      for (int i = 0; i < NQ; ++i) {
+        if (i >= m) continue;
+        const int tt = t + 8 * i;
+        __nv_bfloat16* o = to_k ? ep.kdst + ((size_t)seq_s[tt] * ep.T + pos_s[tt]) * ep.G * ep.head_dim + (n0 - ep.k_col0)
+                                : static_cast<__nv_bfloat16*>(ep.out) + (size_t)tt * ep.ldo + n0;
+        store_bf16x4(o + r0, x[i].x * c[i].x - y[i].x * c[i].y, x[i].y * c[i].z - y[i].y * c[i].w,
+                     x[i].z * d[i].x - y[i].z * d[i].y, x[i].w * d[i].z - y[i].w * d[i].w);
+        store_bf16x4(o + r1, y[i].x * c[i].x + x[i].x * c[i].y, y[i].y * c[i].z + x[i].y * c[i].w,
+                     y[i].z * d[i].x + x[i].z * d[i].y, y[i].w * d[i].z + x[i].w * d[i].w);
+      }
+    }
+  }
+}
+
+template <int EPI>
+__global__ void __launch_bounds__(FW_THREADS, 2)
+    few_gemm_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
+                    const __grid_constant__ FewArgs a, int* err) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base - raw);
+  const uint32_t bars = base + FW_RING;
+  const uint32_t full0 = bars, empty0 = bars + 8 * FW_MAX_STAGES, done = empty0 + 8 * FW_MAX_STAGES, holder = done + 8;
+  volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
+  int* pos_s = reinterpret_cast<int*>(smem + FW_RING + 256);
+  int* seq_s = pos_s + FEW_MAX_ROWS;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int S = (int)cluster_size(), rank = (int)cluster_rank();
+  const int u = (int)blockIdx.x / S;  // the cluster's tile
+  const int kb0 = rank * a.nkb / S, nkb = (rank + 1) * a.nkb / S - kb0;
+  // a stage: the weight rows of one K block, then the tokens'.  The stage pitch is that of
+  // the most tokens the launch may hold, known before the row count is.
+  const int stage_bytes = FW_W_BYTES + a.nt_max * 128;
+  const int stages = min(FW_RING / stage_bytes, FW_MAX_STAGES);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < stages; ++s) {
+      mbar_init(full0 + 8 * s, 1);
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(done, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tmap(&tw);
+    prefetch_tmap(&tx);
+  }
+
+  auto load_w = [&](int stage, int kb) {
+    const uint32_t dst = base + (uint32_t)(stage * stage_bytes), bar = full0 + 8 * stage;
+    if constexpr (EPI == EPI_SWIGLU) {  // 64 gate rows and the matching 64 up rows (128 rows apart)
+      const int row = (u >> 1) * 256 + (u & 1) * 64;
+      tma_load_2d(dst, &tw, (kb0 + kb) * FW_BK, row, bar);
+      tma_load_2d(dst + FW_W_BYTES / 2, &tw, (kb0 + kb) * FW_BK, row + 128, bar);
+    } else {
+      tma_load_2d(dst, &tw, (kb0 + kb) * FW_BK, u * FW_TILE, bar);
+    }
+  };
+  // the first stages' weights, before the dependent-launch wait (no kernel of the step writes them)
+  int pre = 0;
+  if (a.ep.w_early && threadIdx.x == 0)
+    for (; pre < stages && pre < nkb; ++pre) {
+      mbar_expect_tx(full0 + 8 * pre, FW_W_BYTES);
+      load_w(pre, pre);
+    }
+  if (warp == 1) tmem_alloc(holder, FEW_MAX_ROWS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *holder_ptr;
+
+  pdl_wait();
+  pdl_launch_dependents();
+  const int rows = a.ep.m_dev ? min(a.M, *a.ep.m_dev) : a.M;
+  int nt = (rows + 31) & ~31;  // the MMA's N
+  if (nt > a.nt_max) {         // (the launch is not chosen for so many rows)
+    if (threadIdx.x == 0) report_error(err, DERR_BAD_SHAPE);
+    nt = 0;
+  }
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ------------------------------------------------ TMA producer
+      bool ok = true;
+      int issued = 0;
+      for (int kb = 0; kb < (nt > 0 ? nkb : pre); ++kb) {
+        const int stage = kb % stages;
+        const bool have_w = kb < pre;
+        if (!have_w && !mbar_wait(empty0 + 8 * stage, ((uint32_t)(kb / stages) & 1u) ^ 1u, abort_flag)) {
+          ok = false;
+          break;
+        }
+        mbar_arrive_expect_tx(full0 + 8 * stage, (have_w ? 0 : FW_W_BYTES) + nt * 128);
+        if (!have_w) load_w(stage, kb);
+        for (int b = 0; b < nt / 32; ++b)
+          tma_load_2d(base + (uint32_t)(stage * stage_bytes + FW_W_BYTES + b * FW_XBOX_BYTES), &tx, (kb0 + kb) * FW_BK,
+                      b * 32, full0 + 8 * stage);
+        ++issued;
+      }
+      if (!ok) {
+        *abort_flag = 1;
+        report_error(err, DERR_WAIT_TIMEOUT);
+      }
+      if (!ok || nt == 0) {  // every copy issued lands before the CTA leaves (bounded)
+        for (int s = 0; s < stages && s < issued; ++s) {
+          const int arms = (issued - 1 - s) / stages + 1;
+          volatile int no_abort = 0;
+          mbar_wait(full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && nt > 0) {
+      // ------------------------------------------------ MMA issuer
+      const uint32_t idesc = make_idesc(FW_TILE, nt);
+      bool ok = true;
+      for (int kb = 0; kb < nkb; ++kb) {
+        const int stage = kb % stages;
+        if (!mbar_wait(full0 + 8 * stage, (uint32_t)(kb / stages) & 1u, abort_flag)) {
+          ok = false;
+          break;
+        }
+        const uint32_t sw = base + (uint32_t)(stage * stage_bytes);
+        const uint64_t dw = sw128_desc(sw), dx = sw128_desc(sw + FW_W_BYTES);
+#pragma unroll
+        for (int k = 0; k < FW_BK / 16; ++k)
+          umma_bf16(tmem_base, dw + 2 * k, dx + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        umma_commit(empty0 + 8 * stage);
+      }
+      if (!ok) {
+        *abort_flag = 1;
+        report_error(err, DERR_WAIT_TIMEOUT);
+      }
+      umma_commit(done);  // (in either case every MMA issued here completes before TMEM is released)
+      volatile int no_abort = 0;
+      mbar_wait(done, 0, &no_abort);
+    }
+  } else if (nt > 0) {
+    // ------------------------------------------------ epilogue warps 2..5: the sum to shared memory
+    const int et = threadIdx.x - 64;
+    if (EPI == EPI_QKV_ROPE && et < rows) {
+      pos_s[et] = a.ep.row_pos[et];
+      seq_s[et] = a.ep.row_seq[et];
+    }
+    const int q = warp & 3;  // TMEM lane quarter: rows 32 q .. 32 q + 31 of the tile
+    bool ok = mbar_wait(done, 0, abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    if (!ok) {
+      *abort_flag = 1;
+      report_error(err, DERR_WAIT_TIMEOUT);
+    } else {
+      tc_fence_after();
+#pragma unroll 1
+      for (int t0 = 0; t0 < nt; t0 += 32) {
+        uint32_t v[32];
+        tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)t0, v);
+        tmem_ld_wait();
+        const uint32_t at = base + (uint32_t)(t0 * FW_PITCH + q * 32 + lane) * 4;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) st_shared_f32(at + (uint32_t)(i * FW_PITCH * 4), f32(v[i]));
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    tmem_dealloc(tmem_base, FEW_MAX_ROWS);
+  }
+  if (S > 1) cluster_sync();  // every CTA of the cluster has its sum in shared memory
+  if (warp >= 2 && nt > 0 && !*abort_flag) {
+    const int t0 = rank * nt / S, t1 = min((rank + 1) * nt / S, rows);
+    const int et = threadIdx.x - 64;
+    switch (S) {
+      case 1: few_finish<EPI, 1>(a, base, u, t0, t1, et, pos_s, seq_s); break;
+      case 2: few_finish<EPI, 2>(a, base, u, t0, t1, et, pos_s, seq_s); break;
+      case 4: few_finish<EPI, 4>(a, base, u, t0, t1, et, pos_s, seq_s); break;
+      case 8: few_finish<EPI, 8>(a, base, u, t0, t1, et, pos_s, seq_s); break;
+    }
+  }
+  __syncwarp();
+  if (S > 1) cluster_sync_relaxed();  // no CTA leaves while another may read its sum
+}
+
+bool encode_2d(CUtensorMap* tm, const void* p, int rows, int k, int box_rows) {
+  const uint64_t dims[2] = {(uint64_t)k, (uint64_t)rows};
+  const uint64_t strides[1] = {(uint64_t)k * 2};
+  const uint32_t box[2] = {FW_BK, (uint32_t)box_rows};
+  return encode_tmap(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(p), dims, strides, box,
+                     CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+template <int EPI>
+cudaError_t launch_few(const FewPlan& p, int* err, cudaStream_t stream) {
+  static bool attr_set = false;
+  auto kern = few_gemm_kernel<EPI>;
+  if (!attr_set) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FW_SMEM);
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
+  FewArgs a;
+  a.nkb = p.K / FW_BK;
+  a.nt_max = p.nt_max;
+  a.N = p.N;
+  a.M = p.M;
+  a.ep = p.ep;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(p.units * p.split);
+  cfg.blockDim = dim3(FW_THREADS);
+  cfg.dynamicSmemBytes = FW_SMEM;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = p.split;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, p.tw, p.tx, a, err);
+}
+
+}  // namespace
+
+cudaError_t few_plan(FewPlan* p, const void* X, int M, int K, const void* W, int N, int epi, const FewEpi& ep,
+                     int num_sms, int nt_max) {
+  if (M <= 0 || N <= 0 || K <= 0 || K % FW_BK || (nt_max != 32 && nt_max != FEW_MAX_ROWS)) return cudaErrorInvalidValue;
+  if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(W) & 15) ||
+      (reinterpret_cast<uintptr_t>(ep.out) & 15) || ep.ldo % 4 || N % 4)
+    return cudaErrorInvalidValue;
+  switch (epi) {
+    case EPI_BF16:
+    case EPI_RESID_F32: break;
+    case EPI_SWIGLU:
+      if (N % 256) return cudaErrorInvalidValue;
+      break;
+    case EPI_QKV_ROPE:  // whole heads in a tile, each tile all q, all k or all v
+      if ((ep.head_dim != 64 && ep.head_dim != 128) || ep.rope_cols % FW_TILE || N % ep.head_dim ||
+          (ep.kdst && ep.k_col0 % FW_TILE))
+        return cudaErrorInvalidValue;
+      break;
+    default: return cudaErrorInvalidValue;
+  }
+  if (!encode_2d(&p->tw, W, N, K, epi == EPI_SWIGLU ? FW_TILE / 2 : FW_TILE) || !encode_2d(&p->tx, X, M, K, 32))
+    return cudaErrorInvalidValue;
+  p->M = M;
+  p->N = N;
+  p->K = K;
+  p->epi = epi;
+  p->ep = ep;
+  p->nt_max = nt_max;
+  p->units = (N + FW_TILE - 1) / FW_TILE;
+  p->split = 1;
+  while (p->split < 8 && p->units * p->split * 2 <= 2 * num_sms && K / FW_BK / (p->split * 2) >= 1) p->split *= 2;
+  return cudaSuccess;
+}
+
+cudaError_t few_launch(const FewPlan& p, int* err, cudaStream_t stream) {
+  switch (p.epi) {
+    case EPI_BF16: return launch_few<EPI_BF16>(p, err, stream);
+    case EPI_RESID_F32: return launch_few<EPI_RESID_F32>(p, err, stream);
+    case EPI_QKV_ROPE: return launch_few<EPI_QKV_ROPE>(p, err, stream);
+    case EPI_SWIGLU: return launch_few<EPI_SWIGLU>(p, err, stream);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace dcl

@@ -18,70 +18,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// ------------------------------------------------------------------ step row plan
-// One CTA: per sequence the first computed position (0 under full recompute and on a cache
-// refresh, the block-aligned prefix end N + Bk*floor((p-N)/Bk) when the stored keys and
-// values are that block's, T for a finished row), the row offsets, and the row tables.
-__global__ void __launch_bounds__(1024) row_plan_kernel(RowPlan rp, const int32_t* __restrict__ p, int B, int N,
-                                                        int T, int Bk, int cached, int update,
-                                                        int32_t* __restrict__ x, int window, int mask_id) {
-  pdl_wait();
-  pdl_launch_dependents();
-  extern __shared__ int lm_off[];  // [B], then the sequences' first computed positions [B]
-  int* st_pos = lm_off + B;
-  const int M = T - N;
-  if (threadIdx.x == 0) {
-    int off = 0, lmoff = 0;
-    for (int b = 0; b < B; ++b) {
-      const int pb = p[b];
-      int start, end = T, cap = T;
-      if (pb >= T) {
-        start = T;
-      } else if (!cached) {
-        start = 0;
-      } else {
-        const int pe = N + Bk * ((pb - N) / Bk);
-        start = (rp.pe_cache[b] == pe) ? pe : 0;
-        if (update) rp.pe_cache[b] = pe;
-        if (cached == 2 && start != 0) {  // dual cache between refreshes: the current block
-          end = min(pe + Bk, T);
-          cap = end - pb;
-        }
-      }
-      rp.seq_off[b] = off;
-      rp.seq_len[b] = end - start;
-      rp.kcap[b] = cap;
-      st_pos[b] = start;
-      off += end - start;
-      lm_off[b] = lmoff;
-      lmoff += max(end - max(start, N), 0);
-    }
-    rp.counts[0] = off;
-    rp.counts[1] = lmoff;
-  }
-  __syncthreads();
-  for (int b = 0; b < B; ++b) {
-    const int len = rp.seq_len[b], off = rp.seq_off[b], start = st_pos[b], end = start + len;
-    for (int i = threadIdx.x; i < len; i += blockDim.x) {
-      rp.row_seq[off + i] = b;
-      rp.row_pos[off + i] = start + i;
-    }
-    if (cached == 2 && window > 0 && p[b] < T) {
-      // Eq. remasking over the window positions past the computed rows (the embedding
-      // kernel re-masks the computed ones): between refreshes of the dual cache the window
-      // runs past the block
-      const int pb = p[b], w0 = max(pb, end), w1 = min(pb + window, T);
-      for (int t = w0 + threadIdx.x; t < w1; t += blockDim.x) x[(size_t)b * T + t] = mask_id;
-    }
-    const int s0 = max(start, N);
-    for (int i = threadIdx.x; i < end - s0; i += blockDim.x) {
-      const int pos = s0 + i;
-      rp.lm_src[lm_off[b] + i] = off + (pos - start);
-      rp.lm_slot[lm_off[b] + i] = b * M + (pos - N);
-    }
-  }
-}
-
 // ------------------------------------------------------------------ embedding + remask
 // Row r of the step (grid: the most rows a step can have) is position row_pos[r] of
 // sequence row_seq[r]; rows past the step's count return.
@@ -124,9 +60,10 @@ __global__ void __launch_bounds__(THREADS) rmsnorm_kernel(const float* __restric
                                                           const __nv_bfloat16* __restrict__ gain,
                                                           __nv_bfloat16* __restrict__ y, int d,
                                                           float eps, const int* __restrict__ rows_dev,
-                                                          const int* __restrict__ src) {
+                                                          const int* __restrict__ src, int early) {
+  if (early) pdl_launch_dependents();
   pdl_wait();
-  pdl_launch_dependents();
+  if (!early) pdl_launch_dependents();
   const int r = blockIdx.x;
   if (rows_dev && r >= *rows_dev) return;
   const int in_row = src ? src[r] : r;
@@ -165,9 +102,10 @@ __global__ void __launch_bounds__(THREADS) rmsnorm_kernel(const float* __restric
 template <int VPT, int ROWS>
 __global__ void __launch_bounds__(128 * ROWS) rmsnorm_reg_kernel(
     const float* __restrict__ x, const __nv_bfloat16* __restrict__ gain, __nv_bfloat16* __restrict__ y,
-    int rows, int d, float eps, const int* __restrict__ rows_dev, const int* __restrict__ src) {
+    int rows, int d, float eps, const int* __restrict__ rows_dev, const int* __restrict__ src, int early) {
+  if (early) pdl_launch_dependents();
   pdl_wait();
-  pdl_launch_dependents();
+  if (!early) pdl_launch_dependents();
   if (rows_dev) rows = min(rows, *rows_dev);
   const int sub = threadIdx.x >> 7, t = threadIdx.x & 127;
   const int r = blockIdx.x * ROWS + sub;
@@ -722,14 +660,6 @@ __global__ void generate_kernel(__nv_bfloat16* __restrict__ dst, uint64_t seed, 
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
-cudaError_t row_plan_launch(const RowPlan& rp, const int32_t* p, int batch, int N, int T, int block_len, int cached,
-                            int update, int32_t* x, int window, int mask_id, cudaStream_t stream) {
-  if (batch <= 0 || batch > 4096 || (cached && block_len <= 0) || cached < 0 || cached > 2 || (cached == 2 && !x))
-    return cudaErrorInvalidValue;
-  return launch_pdl(row_plan_kernel, 1, 1024, 2 * sizeof(int) * batch, stream, rp, p, batch, N, T, block_len, cached,
-                    update, x, window, mask_id);
-}
-
 cudaError_t embed_remask_launch(int32_t* x, const int32_t* p, int batch, int T, int window,
                                 int mask_id, int vocab, const __nv_bfloat16* embed, int d, float* h,
                                 int* err, const RowPlan& rp, cudaStream_t stream) {
@@ -739,18 +669,18 @@ cudaError_t embed_remask_launch(int32_t* x, const int32_t* p, int batch, int T, 
 }
 
 cudaError_t rmsnorm_launch(const float* x, const __nv_bfloat16* gain, __nv_bfloat16* y, int rows, int d,
-                           float eps, const int* rows_dev, const int* src, cudaStream_t stream) {
+                           float eps, const int* rows_dev, const int* src, bool early, cudaStream_t stream) {
   if (d % 4 || rows <= 0) return cudaErrorInvalidValue;
   const int vpt = (d / 4 + 127) / 128;  // float4 per thread with 128 threads per row
   const int grid2 = (rows + 1) / 2;
   switch (vpt) {
-    case 1: return launch_pdl(rmsnorm_reg_kernel<1, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src);
-    case 2: return launch_pdl(rmsnorm_reg_kernel<2, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src);
-    case 4: case 3: return launch_pdl(rmsnorm_reg_kernel<4, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src);
+    case 1: return launch_pdl(rmsnorm_reg_kernel<1, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src, (int)early);
+    case 2: return launch_pdl(rmsnorm_reg_kernel<2, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src, (int)early);
+    case 4: case 3: return launch_pdl(rmsnorm_reg_kernel<4, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src, (int)early);
     case 5: case 6: case 7: case 8:
-      return launch_pdl(rmsnorm_reg_kernel<8, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src);
+      return launch_pdl(rmsnorm_reg_kernel<8, 2>, grid2, 256, 0, stream, x, gain, y, rows, d, eps, rows_dev, src, (int)early);
     default:
-      return launch_pdl(rmsnorm_kernel<256>, rows, 256, 0, stream, x, gain, y, d, eps, rows_dev, src);
+      return launch_pdl(rmsnorm_kernel<256>, rows, 256, 0, stream, x, gain, y, d, eps, rows_dev, src, (int)early);
   }
 }
 
@@ -801,22 +731,25 @@ cudaError_t generate_launch(__nv_bfloat16* dst, uint64_t seed, int tid, int64_t 
   return cudaGetLastError();
 }
 
-cudaError_t rope_table_build(float* cos_dev, float* sin_dev, int T, int hd, float theta,
+cudaError_t rope_table_build(float* cos_dev, float* sin_dev, float2* cs_dev, int T, int hd, float theta,
                              cudaStream_t stream) {
   const int half = hd / 2;
+  const size_t n = (size_t)T * half;
   float* hc = nullptr;
-  cudaError_t e = cudaMallocHost(&hc, sizeof(float) * 2 * (size_t)T * half);
+  cudaError_t e = cudaMallocHost(&hc, sizeof(float) * 4 * n);
   if (e != cudaSuccess) return e;
+  float2* cs = reinterpret_cast<float2*>(hc + 2 * n);
   for (int t = 0; t < T; ++t)
     for (int j = 0; j < half; ++j) {
       const double ang = (double)t * pow((double)theta, -2.0 * j / hd);
-      hc[(size_t)j * T + t] = (float)cos(ang);  // [half][T]: positions contiguous
-      hc[(size_t)T * half + (size_t)j * T + t] = (float)sin(ang);
+      const float c = (float)cos(ang), sn = (float)sin(ang);
+      hc[(size_t)j * T + t] = c;  // [half][T]: positions contiguous
+      hc[n + (size_t)j * T + t] = sn;
+      cs[(size_t)t * half + j] = make_float2(c, sn);
     }
-  e = cudaMemcpyAsync(cos_dev, hc, sizeof(float) * (size_t)T * half, cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(sin_dev, hc + (size_t)T * half, sizeof(float) * (size_t)T * half,
-                        cudaMemcpyHostToDevice, stream);
+  e = cudaMemcpyAsync(cos_dev, hc, sizeof(float) * n, cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(sin_dev, hc + n, sizeof(float) * n, cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cs_dev, cs, sizeof(float2) * n, cudaMemcpyHostToDevice, stream);
   cudaError_t s = cudaStreamSynchronize(stream);
   cudaFreeHost(hc);
   return e != cudaSuccess ? e : s;
