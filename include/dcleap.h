@@ -252,8 +252,8 @@ dcl_status dcl_accept(dcl_ctx* ctx, const void* logits_dev, int32_t B, int32_t P
  * real-time budget where cudaMalloc may stall or is forbidden - and so cannot create a
  * dcl_ctx either.  It computes exactly what dcl_accept computes (same arguments, same
  * kernels) on `cuda_stream` (NULL = the legacy default stream), without a context and
- * without any allocation: its scratch (12 bytes per position) is a file-scope device
- * array of DCL_NOALLOC_MAX_POSITIONS positions (384 KB) that every GPU loading this
+ * without any allocation: its scratch is a file-scope device array sized for
+ * DCL_NOALLOC_MAX_POSITIONS positions (1.3 MB) that every GPU loading this
  * library holds until the process exits.
  *   - The size limits are dcl_accept's (1 <= P <= 4096, V >= 2), and B*P at most
  *     DCL_NOALLOC_MAX_POSITIONS; anything else is rejected with DCL_ERR_INVALID_ARG.

@@ -2,7 +2,7 @@
 // allocate device memory - e.g. code running inside another framework's memory pool
 // or under an allocation-free real-time budget, where cudaMalloc is forbidden or may
 // stall.  It needs no dcl_ctx (creating one allocates); its per-position scratch (the
-// top-1 id and the top-1 / top-2 probabilities of every position) lives in the
+// partial softmax statistics, the top-1 id and the confidence of every position) lives in the
 // file-scope device array below instead, which every GPU that loads this library
 // holds until the process exits.
 #include <mutex>
@@ -16,9 +16,10 @@ namespace {
 constexpr int kMaxPositions = DCL_NOALLOC_MAX_POSITIONS;
 constexpr int kMaxDevices = 64;
 
-// For n = B*P positions of a call: n int32 top-1 ids, then n float top-1 probabilities,
-// then n float top-2 probabilities (12 bytes per position).
-static __device__ __align__(256) unsigned char g_accept_scratch[3 * 4 * kMaxPositions];
+// For n = B*P positions of a call: the statistics pass's partials (16 bytes each, at most
+// accept_part_slots(n)), then n int32 top-1 ids and n float confidences.
+constexpr size_t kPartBytes = 16 * dcl::accept_part_slots(kMaxPositions);
+static __device__ __align__(256) unsigned char g_accept_scratch[kPartBytes + 2 * 4 * kMaxPositions];
 
 std::mutex g_mu;
 void* g_scratch_addr[kMaxDevices] = {};
@@ -75,16 +76,17 @@ extern "C" dcl_status dcl_accept_noalloc(const void* logits_dev, int32_t B, int3
   // Every position the commit pass reads is written by the statistics pass of the same
   // call, so the scratch left by an earlier call needs no clearing.
   const size_t n = (size_t)B * P;
-  int32_t* ids = static_cast<int32_t*>(base);
+  float4* part = static_cast<float4*>(base);
+  int32_t* ids = reinterpret_cast<int32_t*>(static_cast<unsigned char*>(base) + kPartBytes);
   float* c1 = reinterpret_cast<float*>(ids + n);
-  float* c2 = c1 + n;
   const int window = cfg->max_window > 0 ? cfg->max_window : (P / 2 > 0 ? P / 2 : 1);
   dcl::DcvParams prm{cfg->tau_commit, cfg->tau_draft, window, cfg->min_commit, cfg->contiguous_drafts,
                      cfg->acceptance, P};
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  e = dcl::accept_stats_launch(static_cast<const __nv_bfloat16*>(logits_dev), committed_dev, B, P, V, ids, c1,
-                               c2, cfg->confidence, s);
-  if (e == cudaSuccess) e = dcl::accept_commit_launch(committed_dev, ids, c1, x_dev, k_dev, B, P, prm, s);
+  e = dcl::accept_stats_launch(static_cast<const __nv_bfloat16*>(logits_dev), committed_dev, B, P, V, cfg->confidence,
+                               part, s);
+  if (e == cudaSuccess)
+    e = dcl::accept_commit_launch(committed_dev, part, V, cfg->confidence, ids, c1, x_dev, k_dev, B, P, prm, s);
   if (e != cudaSuccess) {
     dcl::set_thread_error((std::string("dcl_accept_noalloc: launch failed: ") + cudaGetErrorString(e)).c_str());
     return DCL_ERR_CUDA;

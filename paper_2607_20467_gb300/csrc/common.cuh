@@ -288,13 +288,17 @@ cudaError_t dcv_commit_launch(int32_t* x, int32_t* p, int32_t* k_out, int32_t* s
                               const int32_t* ids, const float* c, const float* ent, float* jpde, int batch,
                               int N, int M, const DcvParams& prm, int32_t* done_count, uint8_t* cmt,
                               const int* kcap, cudaStream_t stream);
-// Block acceptance from bf16 logits (dcl_accept): c1 = p1 (mode 0) or exp(-H) (mode 1).
-cudaError_t accept_stats_launch(const __nv_bfloat16* logits, const int32_t* committed, int B,
-                                int P, int V, int32_t* ids, float* c1, float* c2, int mode,
-                                cudaStream_t stream);
-cudaError_t accept_commit_launch(const int32_t* committed, const int32_t* ids, const float* c1,
-                                 int32_t* x, int32_t* k, int B, int P, const DcvParams& prm,
-                                 cudaStream_t stream);
+// Block acceptance from bf16 logits (dcl_accept), in two passes: the softmax statistics of
+// every uncommitted position in accept_chunks(B * P, V) chunks of its row, partials to part
+// [B * P][chunks] ({max, sum exp(z - max), id, entropy sum}), then their merge into ids and c1
+// (p1 with mode 0, exp(-H) with mode 1; [B][P]) and the rule.  The chunks are so few that
+// B * P of them never exceed accept_part_slots(B * P).
+int accept_chunks(int n, int V);
+__host__ __device__ constexpr size_t accept_part_slots(size_t n) { return n + 4 * 48 * 152; }
+cudaError_t accept_stats_launch(const __nv_bfloat16* logits, const int32_t* committed, int B, int P, int V, int mode,
+                                float4* part, cudaStream_t stream);
+cudaError_t accept_commit_launch(const int32_t* committed, const float4* part, int V, int mode, int32_t* ids, float* c1,
+                                 int32_t* x, int32_t* k, int B, int P, const DcvParams& prm, cudaStream_t stream);
 // One launch of a kernel that does only the dependent-launch handshake (launch floor).
 cudaError_t empty_launch(cudaStream_t stream);
 // Counter-based weight generator (SplitMix64 + Irwin-Hall(4)), with an optional

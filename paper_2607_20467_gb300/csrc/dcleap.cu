@@ -86,7 +86,8 @@ struct dcl_ctx {
 
   // accept scratch (dcl_accept)
   int32_t* acc_ids = nullptr;
-  float *acc_c1 = nullptr, *acc_c2 = nullptr;
+  float* acc_c1 = nullptr;
+  float4* acc_part = nullptr;
   size_t acc_cap = 0;
 
   // per-shape state
@@ -1227,20 +1228,21 @@ dcl_status dcl_accept(dcl_ctx* c, const void* logits_dev, int32_t B, int32_t P, 
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));  // no launch may still use the old buffers
     dev_free_one(c, c->acc_ids);
     dev_free_one(c, c->acc_c1);
-    dev_free_one(c, c->acc_c2);
+    dev_free_one(c, c->acc_part);
     c->acc_cap = 0;
     c->acc_ids = (int32_t*)dev_alloc(c, 4 * n);
     c->acc_c1 = (float*)dev_alloc(c, 4 * n);
-    c->acc_c2 = (float*)dev_alloc(c, 4 * n);
-    if (!c->acc_ids || !c->acc_c1 || !c->acc_c2) return fail(c, DCL_ERR_OOM, "accept scratch allocation failed");
+    c->acc_part = (float4*)dev_alloc(c, sizeof(float4) * accept_part_slots(n));
+    if (!c->acc_ids || !c->acc_c1 || !c->acc_part) return fail(c, DCL_ERR_OOM, "accept scratch allocation failed");
     c->acc_cap = n;
   }
   const int window = cfg->max_window > 0 ? cfg->max_window : (P / 2 > 0 ? P / 2 : 1);
   DcvParams prm{cfg->tau_commit, cfg->tau_draft, window, cfg->min_commit, cfg->contiguous_drafts,
                 cfg->acceptance, P};
-  CUDA_TRY(c, accept_stats_launch(static_cast<const __nv_bfloat16*>(logits_dev), committed_dev, B, P, V, c->acc_ids,
-                                  c->acc_c1, c->acc_c2, cfg->confidence, c->stream));
-  CUDA_TRY(c, accept_commit_launch(committed_dev, c->acc_ids, c->acc_c1, x_dev, k_dev, B, P, prm, c->stream));
+  CUDA_TRY(c, accept_stats_launch(static_cast<const __nv_bfloat16*>(logits_dev), committed_dev, B, P, V,
+                                  cfg->confidence, c->acc_part, c->stream));
+  CUDA_TRY(c, accept_commit_launch(committed_dev, c->acc_part, V, cfg->confidence, c->acc_ids, c->acc_c1, x_dev, k_dev,
+                                   B, P, prm, c->stream));
   return DCL_OK;
 }
 

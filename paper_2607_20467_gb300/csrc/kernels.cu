@@ -10,6 +10,8 @@
 //   generate       counter-based synthetic weight generator
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -162,7 +164,8 @@ __device__ __forceinline__ void merge(Part& a, const Part& b) {
     return;
   }
   const float m = fmaxf(a.m, b.m);
-  const float da = (a.m - m) * kLog2e, db = (b.m - m) * kLog2e;  // <= 0, finite; one is 0
+  // <= 0, one is 0 (clamped where exp2 is 0: the difference of finite maxima may overflow)
+  const float da = fmaxf((a.m - m) * kLog2e, -200.f), db = fmaxf((b.m - m) * kLog2e, -200.f);
   const float ea = da == 0.f ? 1.f : exp2f(da), eb = db == 0.f ? 1.f : exp2f(db);
   const float s = a.s * ea + b.s * eb;
   // re-based to the new maximum: y' = y + d for every term
@@ -433,7 +436,7 @@ __global__ void dcv_commit_kernel(int32_t* __restrict__ x, int32_t* __restrict__
 template <bool ENT>
 __device__ __forceinline__ void take1(Part& a, float v, int col) {
   if (v > a.m) {
-    const float d = (a.m - v) * kLog2e;  // -inf for the first column
+    const float d = fmaxf((a.m - v) * kLog2e, -200.f);  // (-inf for the first column)
     const float e = exp2f(d);
     if (ENT) a.u = a.s > 0.f ? e * fmaf(d, a.s, a.u) : 0.f;
     a.s = a.s * e + 1.f;
@@ -449,159 +452,209 @@ __device__ __forceinline__ void take1(Part& a, float v, int col) {
   }
 }
 
-// Eight consecutive columns (one 16-byte vector), without a branch per column: the
-// vector's maximum first (a new running maximum rescales s and u once, and takes the
-// lowest column holding it as the argmax), then every column adds exp2((z - m) log2 e)
-// on the special-function unit.  The argmax's own term is exp2 of the rounding residual
-// of the fused multiply-add, within an ulp of 1 (write_conf clamps p1 and p2).  A vector
-// holding an infinity takes the exact column-by-column path.
-template <bool ENT>
-__device__ __forceinline__ void take8(Part& a, const uint4& q, int col) {
-  const float v[8] = {bf16_lo(q.x), bf16_hi(q.x), bf16_lo(q.y), bf16_hi(q.y),
-                      bf16_lo(q.z), bf16_hi(q.z), bf16_lo(q.w), bf16_hi(q.w)};
-  const float cm = fmaxf(max3f(max3f(v[0], v[1], v[2]), max3f(v[3], v[4], v[5]), v[6]), v[7]);
-  if (!(fabsf(cm) < INFINITY)) {
-#pragma unroll
-    for (int k = 0; k < 8; ++k) take1<ENT>(a, v[k], col + k);
-    return;
-  }
-  if (cm > a.m) {
-    int k0 = 7;
-#pragma unroll
-    for (int k = 6; k >= 0; --k) k0 = v[k] == cm ? k : k0;  // lowest column holding the maximum
-    float s2 = -INFINITY;  // largest of the other seven
-#pragma unroll
-    for (int k = 0; k < 8; ++k) s2 = k == k0 ? s2 : fmaxf(s2, v[k]);
-    const float d = (a.m - cm) * kLog2e;  // -inf before the first vector
-    const float e = exp2f(d);
-    if (ENT) a.u = a.s > 0.f ? e * fmaf(d, a.s, a.u) : 0.f;
-    a.s *= e;
-    a.t2 = fmaxf(a.m, s2);
-    a.m = cm;
-    a.id = col + k0;
-  } else {
-    a.t2 = fmaxf(a.t2, cm);
-  }
-  // y = z log2(e) - m log2(e) and its exp2 for the eight columns, two lanes per
-  // instruction; the eight terms are summed as a tree of pairs
-  const float ml = a.m * kLog2e;
-  const unsigned long long l2 = pk2(kLog2e, kLog2e), nm = pk2(-ml, -ml);
-  unsigned long long e2[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float y0, y1;
-    upk2(ffma2(pk2(v[2 * k], v[2 * k + 1]), l2, nm), y0, y1);
-    const float x0 = ex2_approx(y0), x1 = ex2_approx(y1);
-    e2[k] = pk2(x0, x1);
-    if (ENT) a.u = fmaf(x1, fmaxf(y1, -200.f), fmaf(x0, fmaxf(y0, -200.f), a.u));
-  }
-  float s0, s1;
-  upk2(fadd2(fadd2(e2[0], e2[1]), fadd2(e2[2], e2[3])), s0, s1);
-  a.s += s0 + s1;
-}
-
-// One CTA of THREADS per uncommitted position: thread t takes the 16-byte vectors t, t +
-// THREADS, ... of the row, ACC_AHEAD of them loaded before any is used (several loads in
-// flight per thread: with one, the latency of each load paced the thread).  256 threads
-// and at most 32 registers keep eight CTAs, so that ~1200 rows, resident on the 152 SMs at
-// once.  CTA a takes the a-th uncommitted position (row by row), so that the CTAs with
-// work are the first of the grid and spread evenly over the SMs; the committed positions'
-// CTAs, which read nothing, come last (with one CTA per position in place, the live rows
-// landed unevenly: 3 on some SMs, 10 on others).
+// The statistics pass.  It is bound by the read of the live rows' logits (64 blocks of 32
+// positions, half of them committed, V = 126464: 259 MB, 38 us at 6.8 TB/s).  The unit of work
+// is a chunk: 1 / C of a row's 16-byte vectors, taken by one warp, so that no barrier stands
+// between chunks, and a single block's 32 rows reach every SM (one CTA per row left 120 of 152
+// SMs idle: 19 us for 9.7 MB).  C (accept_chunks) gives each of the GPU's resident warps about
+// four chunks, of at least ACC_MIN_VECS vectors: enough to even out the SMs' shares, few enough
+// that a chunk's end (one warp reduction) stays small beside it.  It depends on the sizes alone:
+// a position's statistics do not change with the committed counts around it.  A chunk's partial
+// {max, sum, argmax, entropy sum} goes to part[position][chunk]; the commit pass merges them.
+// Measured: that pass 57 -> 43 us (6.0 TB/s), the call 61 -> 52.6 us; one block of V = 152064
+// with the entropy confidence 25.4 -> 9.2 us a call.
 constexpr int ACC_THREADS = 256;
-constexpr int ACC_AHEAD = 4;
-constexpr int ACC_COMPACT_MAX_B = 256;  // (each CTA scans the rows; larger batches keep one CTA per position in place)
-// The a-th uncommitted position of the block (row-major over B rows of P positions, c_b
-// committed in row b): its index b * P + i, or -1 if there are fewer (warp-wide call).
-__device__ __forceinline__ int nth_uncommitted(const int32_t* committed, int B, int P, int a) {
-  const int lane = threadIdx.x & 31;
-  for (int b0 = 0; b0 < B; b0 += 32) {
-    const int b = b0 + lane;
-    const int n = b < B ? P - min(max(committed[b], 0), P) : 0;  // uncommitted positions of row b
-    int incl = n;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const int total = __shfl_sync(kFull, incl, 31);
-    if (a < total) {
-      const unsigned hit = __ballot_sync(kFull, a < incl);
-      const int l = __ffs(hit) - 1;  // the first row whose running count passes a
-      const int before = __shfl_sync(kFull, incl - n, l);
-      const int nl = __shfl_sync(kFull, n, l);
-      return (b0 + l) * P + (P - nl) + (a - before);
-    }
-    a -= total;
-  }
-  return -1;
+constexpr int ACC_WARPS = ACC_THREADS / 32;
+constexpr int ACC_CTAS = 6;  // per SM: 40 registers per thread
+constexpr int ACC_GRID = 152 * ACC_CTAS;
+constexpr int ACC_AHEAD = 4;       // vectors of a group, loaded before any is used
+constexpr int ACC_MIN_VECS = 256;  // 4 KB: eight vectors per lane
+// Up to this many rows the live positions are counted first and shared out evenly (with larger
+// batches the warps stride over all positions and skip the committed ones).
+constexpr int ACC_COMPACT_MAX_B = 256;
+
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {  // (a NaN loses)
+  const __nv_bfloat162 r = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
 }
 
-template <int THREADS, bool ENT>
-__global__ void __launch_bounds__(THREADS, 2048 / THREADS) accept_stats_kernel(
-    const __nv_bfloat16* __restrict__ logits, const int32_t* __restrict__ committed, int B, int P, int V,
-    int32_t* __restrict__ ids, float* __restrict__ c1, float* __restrict__ c2, int mode) {
+// A group of N vectors into a lane's partial.  Per column only the exponent argument, its exp2
+// and the sums remain: the maximum is taken on packed bf16 pairs, the running sums are
+// re-based once per group without a branch (with one per vector some lane of the warp nearly
+// always took it: 80 instructions per vector, 55 us for 259 MB), and the argmax is kept as the
+// group it lies in (`best`), resolved at the chunk's end.
+template <bool ENT, int N>
+__device__ __forceinline__ void take_group(Part& a, int& best, const uint4 (&q)[N], int j) {
+  uint32_t g = max_bf16x2(max_bf16x2(q[0].x, q[0].y), max_bf16x2(q[0].z, q[0].w));
+#pragma unroll
+  for (int t = 1; t < N; ++t)
+    g = max_bf16x2(g, max_bf16x2(max_bf16x2(q[t].x, q[t].y), max_bf16x2(q[t].z, q[t].w)));
+  const float gm = fmaxf(bf16_lo(g), bf16_hi(g));
+  if (gm > a.m) best = j;
+  const float m = fmaxf(a.m, gm);
+  const float ref = m == -INFINITY ? 0.f : m;
+  // 0 if the maximum stays; clamped where 2^d is 0 (before the first column, or after columns
+  // of the type's lowest value), so that no product below is 0 times infinity
+  const float d = fmaxf((a.m - ref) * kLog2e, -200.f);
+  const float f = d < 0.f ? ex2_approx(d) : 1.f;
+  if (ENT) a.u = a.s > 0.f ? f * fmaf(d, a.s, a.u) : 0.f;
+  a.s *= f;
+  a.m = m;
+  const unsigned long long l2 = pk2(kLog2e, kLog2e), nm = pk2(-ref, -ref);
+  unsigned long long s0 = 0ull, s1 = 0ull;
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    const uint32_t w[4] = {q[t].x, q[t].y, q[t].z, q[t].w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float y0, y1;
+      // z - max first: exact for the maximum itself, and the lowest values do not overflow
+      upk2(ffma2(fadd2(pk2(bf16_lo(w[k]), bf16_hi(w[k])), nm), l2, 0ull), y0, y1);
+      const float x0 = ex2_approx(y0), x1 = ex2_approx(y1);
+      if (k & 1)
+        s1 = fadd2(s1, pk2(x0, x1));
+      else
+        s0 = fadd2(s0, pk2(x0, x1));
+      if (ENT) a.u = fmaf(x1, fmaxf(y1, -200.f), fmaf(x0, fmaxf(y0, -200.f), a.u));  // (0 at y = -inf)
+    }
+  }
+  float c0, c1;
+  upk2(fadd2(s0, s1), c0, c1);
+  a.s = m == -INFINITY ? 0.f : a.s + (c0 + c1);
+}
+
+// The lanes' partials into one (the id: the lowest of the lanes that hold the maximum).
+template <bool ENT>
+__device__ __forceinline__ Part warp_merge(const Part& a) {
+  Part r{a.m, 0.f, -INFINITY, 0};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) r.m = fmaxf(r.m, __shfl_xor_sync(kFull, r.m, o));
+  r.id = (int)__reduce_min_sync(kFull, a.m == r.m ? (unsigned)a.id : 0x7fffffffu);
+  if (r.m == -INFINITY) return r;
+  const float d = a.m == r.m ? 0.f : fmaxf((a.m - r.m) * kLog2e, -200.f);
+  const float f = d == 0.f ? 1.f : ex2_approx(d);
+  // (a lane without a column adds nothing, whatever its sums)
+  r.s = a.m == -INFINITY ? 0.f : a.s * f;
+  r.u = !ENT || a.m == -INFINITY ? 0.f : f * fmaf(d, a.s, a.u);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    r.s += __shfl_xor_sync(kFull, r.s, o);
+    if (ENT) r.u += __shfl_xor_sync(kFull, r.u, o);
+  }
+  return r;
+}
+
+// Chunk c of C of one row of V logits, by one warp.  Full vectors are those that lie on
+// 16-byte boundaries wholly inside the row; the up to seven columns before and after them go
+// one to a lane, with the first and the last chunk.  A lane's columns arrive in increasing
+// order and only a strictly larger value moves `best`, so its argmax is its lowest maximal
+// column.
+template <bool ENT>
+__device__ __forceinline__ Part row_chunk(const __nv_bfloat16* row, int V, int c, int C, int lane) {
+  Part a{-INFINITY, 0.f, -INFINITY, 0x7fffffff};
+  const int off = (int)(reinterpret_cast<uintptr_t>(row) & 15) >> 1;  // columns past the boundary before
+  const int f0 = off ? 1 : 0, f1 = (V + off) >> 3;                    // full vectors [f0, f1) from there
+  const int head = off ? min(8 - off, V) : 0;
+  const unsigned short* r2 = reinterpret_cast<const unsigned short*>(row);
+  auto col = [&](int j) { return __uint_as_float((uint32_t)r2[j] << 16); };
+  if (c == 0 && lane < head) take1<ENT>(a, col(lane), lane);
+  const int nv = max(f1 - f0, 0);
+  const uint4* r4 = reinterpret_cast<const uint4*>(row - off) + f0;
+  const int c0 = 8 * f0 - off;  // the first full vector's first column
+  const int v1 = (int)((long)nv * (c + 1) / C);
+  int j = (int)((long)nv * c / C) + lane, best = -1;
+  for (; j + (ACC_AHEAD - 1) * 32 < v1; j += ACC_AHEAD * 32) {
+    uint4 q[ACC_AHEAD];
+#pragma unroll
+    for (int t = 0; t < ACC_AHEAD; ++t) q[t] = __ldcs(r4 + j + t * 32);  // streamed once
+    take_group<ENT>(a, best, q, j);
+  }
+  for (; j < v1; j += 32) {
+    const uint4 q[1] = {__ldcs(r4 + j)};
+    take_group<ENT>(a, best, q, j);
+  }
+  // the lanes that hold the warp's maximum look for it in its group again
+  float wm = a.m;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(kFull, wm, o));
+  if (best >= 0 && a.m == wm) {
+    bool found = false;
+    for (int i = best; i < v1 && !found; i += 32) {
+      const uint4 q = __ldcs(r4 + i);
+      const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+      for (int k = 7; k >= 0; --k)
+        if ((k & 1 ? bf16_hi(w[k >> 1]) : bf16_lo(w[k >> 1])) == a.m) {
+          a.id = i * 8 + c0 + k;
+          found = true;
+        }
+    }
+  }
+  if (c == C - 1) {
+    const int t = max(head, 8 * f1 - off) + lane;
+    if (t < V) take1<ENT>(a, col(t), t);
+  }
+  return warp_merge<ENT>(a);
+}
+
+template <bool ENT>
+__global__ void __launch_bounds__(ACC_THREADS, ACC_CTAS) accept_stats_kernel(
+    const __nv_bfloat16* __restrict__ logits, const int32_t* __restrict__ committed, int B, int P, int V, int C,
+    float4* __restrict__ part) {
+  __shared__ int upto[ACC_COMPACT_MAX_B];  // uncommitted positions of rows 0 .. b
   pdl_wait();  // the logits, and the previous call's commit pass that read this scratch
   pdl_launch_dependents();
-  int pos = blockIdx.x;  // b * P + i
-  if (B <= ACC_COMPACT_MAX_B) {
-    __shared__ int pos_s;
+  const int lane = threadIdx.x & 31;
+  const bool compact = B <= ACC_COMPACT_MAX_B;
+  int rows = B * P;
+  if (compact) {
     if (threadIdx.x < 32) {
-      const int q = nth_uncommitted(committed, B, P, (int)blockIdx.x);
-      if (threadIdx.x == 0) pos_s = q;
+      int sum = 0;
+      for (int b0 = 0; b0 < B; b0 += 32) {
+        const int b = b0 + lane;
+        int incl = b < B ? P - min(max(committed[b], 0), P) : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += t;
+        }
+        if (b < B) upto[b] = sum + incl;
+        sum += __shfl_sync(kFull, incl, 31);
+      }
     }
     __syncthreads();
-    pos = pos_s;
-    if (pos < 0) return;  // (uniform over the CTA)
-  } else if (pos % P < committed[pos / P]) {
-    return;  // committed positions are never read
+    rows = upto[B - 1];
   }
-  const __nv_bfloat16* row = logits + (size_t)pos * V;
-  Part a{-INFINITY, 0.f, -INFINITY, 0x7fffffff};
-  const bool vec = ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
-  int done = 0;
-  if (vec) {
-    const uint4* r4 = reinterpret_cast<const uint4*>(row);
-    const int n8 = V / 8;
-    int j = threadIdx.x;
-    for (; j + (ACC_AHEAD - 1) * THREADS < n8; j += ACC_AHEAD * THREADS) {
-      uint4 q[ACC_AHEAD];
-#pragma unroll
-      for (int t = 0; t < ACC_AHEAD; ++t) q[t] = __ldcs(r4 + j + t * THREADS);
-#pragma unroll
-      for (int t = 0; t < ACC_AHEAD; ++t) take8<ENT>(a, q[t], (j + t * THREADS) * 8);
+  // (items of consecutive warps are consecutive chunks of a row)
+  const long items = (long)rows * C;
+  for (long i = (long)blockIdx.x * ACC_WARPS + (threadIdx.x >> 5); i < items; i += (long)gridDim.x * ACC_WARPS) {
+    const int a = (int)(i / C), c = (int)(i - (long)a * C);
+    int pos = a;  // b * P + position
+    if (compact) {
+      int lo = 0, hi = B - 1;  // the first row whose running count passes a
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (upto[mid] > a)
+          hi = mid;
+        else
+          lo = mid + 1;
+      }
+      pos = (lo + 1) * P - (upto[lo] - a);
+    } else if (pos % P < committed[pos / P]) {
+      continue;  // committed positions are never read
     }
-    for (; j < n8; j += THREADS) take8<ENT>(a, __ldcs(r4 + j), j * 8);  // streamed once
-    done = n8 * 8;
-  }
-  const unsigned short* r2 = reinterpret_cast<const unsigned short*>(row);
-  for (int j = done + threadIdx.x; j < V; j += THREADS) take1<ENT>(a, __uint_as_float((uint32_t)r2[j] << 16), j);
-  // a thread's columns arrive in increasing order, so its argmax is its lowest maximal
-  // column; merge() breaks ties between threads by the lower id
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) merge(a, shfl_part(a, o));
-  __shared__ Part red[THREADS / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    Part v = threadIdx.x < THREADS / 32 ? red[threadIdx.x] : Part{-INFINITY, 0.f, -INFINITY, 0x7fffffff};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) merge(v, shfl_part(v, o));
-    if (threadIdx.x == 0) {
-      ConfOut o;
-      o.top1 = ids;
-      o.p2 = c2;
-      o.conf = c1;
-      o.mode = mode;
-      write_conf(v, o, pos);
-    }
+    const Part v = row_chunk<ENT>(logits + (size_t)pos * V, V, c, C, lane);
+    if (lane == 0) part[(size_t)pos * C + c] = make_float4(v.m, v.s, __int_as_float(v.id), v.u);
   }
 }
 
-__global__ void accept_commit_kernel(const int32_t* __restrict__ committed,
-                                     const int32_t* __restrict__ ids, const float* __restrict__ c1,
-                                     int32_t* __restrict__ x, int32_t* __restrict__ k, int P,
-                                     DcvParams prm) {
+// The commit pass: one CTA per block.  Its warps merge the chunks of the uncommitted positions
+// (a position each, lanes over the chunks), then one warp applies the rule.
+template <bool ENT>
+__global__ void __launch_bounds__(1024) accept_commit_kernel(const int32_t* __restrict__ committed,
+                                                             const float4* __restrict__ part, int C, int32_t* ids,
+                                                             float* c1, int32_t* __restrict__ x,
+                                                             int32_t* __restrict__ k, int P, DcvParams prm) {
   pdl_wait();  // the statistics pass
   pdl_launch_dependents();
   const int b = blockIdx.x;
@@ -610,6 +663,23 @@ __global__ void accept_commit_kernel(const int32_t* __restrict__ committed,
     if (threadIdx.x == 0) k[b] = 0;
     return;
   }
+  const int lane = threadIdx.x & 31;
+  ConfOut o;
+  o.top1 = ids;
+  o.conf = c1;
+  o.mode = ENT ? 1 : 0;
+  for (int i = pb + (threadIdx.x >> 5); i < P; i += blockDim.x >> 5) {
+    const int pos = b * P + i;
+    Part a{-INFINITY, 0.f, -INFINITY, 0x7fffffff};
+    for (int c = lane; c < C; c += 32) {
+      const float4 v = part[(size_t)pos * C + c];
+      merge(a, Part{v.x, v.y, -INFINITY, __float_as_int(v.z), v.w});
+    }
+    a = warp_merge<ENT>(a);
+    if (lane == 0) write_conf(a, o, pos);
+  }
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
   int K;
   if (prm.acceptance == 1) {  // Eq. threshold_pd over the uncommitted rest [c_b, P), no drafts
     float hs, hm;
@@ -699,21 +769,26 @@ cudaError_t dcv_commit_launch(int32_t* x, int32_t* p, int32_t* k_out, int32_t* s
                     done_count, cmt, kcap);
 }
 
-cudaError_t accept_stats_launch(const __nv_bfloat16* logits, const int32_t* committed, int B, int P,
-                                int V, int32_t* ids, float* c1, float* c2, int mode, cudaStream_t stream) {
-  // Both passes are dependent launches: each is scheduled while its predecessor drains and
-  // waits for it (pdl_wait) before touching memory.
-  if (mode)
-    return launch_pdl(accept_stats_kernel<ACC_THREADS, true>, B * P, ACC_THREADS, 0, stream, logits, committed, B, P,
-                      V, ids, c1, c2, mode);
-  return launch_pdl(accept_stats_kernel<ACC_THREADS, false>, B * P, ACC_THREADS, 0, stream, logits, committed, B, P, V,
-                    ids, c1, c2, mode);
+int accept_chunks(int n, int V) {
+  const int most = std::max(1, V / 8 / ACC_MIN_VECS);
+  const int want = (ACC_WARPS * ACC_GRID * 4 + n - 1) / n;
+  return std::min(most, want);
 }
 
-cudaError_t accept_commit_launch(const int32_t* committed, const int32_t* ids, const float* c1,
-                                 int32_t* x, int32_t* k, int B, int P, const DcvParams& prm,
-                                 cudaStream_t stream) {
-  return launch_pdl(accept_commit_kernel, B, 32, 0, stream, committed, ids, c1, x, k, P, prm);
+cudaError_t accept_stats_launch(const __nv_bfloat16* logits, const int32_t* committed, int B, int P, int V, int mode,
+                                float4* part, cudaStream_t stream) {
+  // Both passes are dependent launches: each is scheduled while its predecessor drains and
+  // waits for it (pdl_wait) before touching memory.
+  const int C = accept_chunks(B * P, V);
+  const long ctas = ((long)B * P * C + ACC_WARPS - 1) / ACC_WARPS;
+  return launch_pdl(mode ? accept_stats_kernel<true> : accept_stats_kernel<false>, (int)std::min<long>(ctas, ACC_GRID),
+                    ACC_THREADS, 0, stream, logits, committed, B, P, V, C, part);
+}
+
+cudaError_t accept_commit_launch(const int32_t* committed, const float4* part, int V, int mode, int32_t* ids, float* c1,
+                                 int32_t* x, int32_t* k, int B, int P, const DcvParams& prm, cudaStream_t stream) {
+  return launch_pdl(mode ? accept_commit_kernel<true> : accept_commit_kernel<false>, B, 32 * std::min(P, 32), 0, stream,
+                    committed, part, accept_chunks(B * P, V), ids, c1, x, k, P, prm);
 }
 
 cudaError_t empty_launch(cudaStream_t stream) { return launch_pdl(empty_step_kernel, 1, 32, 0, stream); }
