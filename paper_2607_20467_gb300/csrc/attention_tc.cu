@@ -2,47 +2,88 @@
 // every position attends to every position of its sequence), on the tcgen05 tensor
 // cores of sm_103a.
 //
-// One CTA = 128 query rows of one (sequence, head); the key axis is walked once, in
-// blocks of 128: S_j = Q K_j^T into TMEM (double-buffered), then per row a running
-// maximum m, P_j = exp2(S_j * log2(e)/sqrt(hd) - m) with the row sum l kept in fp32, P_j
-// written to shared memory in fp16 (11 significant bits; P <= 2^8), and O += P_j V_j in
-// TMEM with V^T held in fp16 (the bf16 values of v, which fp16 holds exactly).  m moves
-// only when a block's maximum exceeds it by more than 8 (P stays below 2^8); l and O are
-// then scaled by the same factor, so O / l is unchanged.  O / l leaves through TMA.
+// The unit of query work is a band: 32 consecutive query rows of one head.  One CTA takes up
+// to eight bands of one (sequence, kv head), two tiles of four: consecutive rows of a head
+// with multi-head attention, rows of the heads that share the kv head with grouped queries
+// (so a step that computes 32 rows of a sequence loads its keys once for four heads of a tile,
+// not once per head).  The key axis is walked in blocks of 128: S = Q K^T into TMEM per tile,
+// then per row a running maximum m, P = exp2(S * log2(e)/sqrt(hd) - m) with the row sum l kept
+// in fp32, P written to shared memory in fp16 (11 significant bits; P <= 2^8), and O += P V in
+// TMEM with V^T held in fp16 (the bf16 values of v, which fp16 holds exactly).  m moves only
+// when a block's maximum exceeds it by more than 8 (P stays below 2^8); l and O are then scaled
+// by the same factor, so O / l is unchanged.  O / l leaves through TMA.
 //
-// Roles (320 threads): warp 0 lane 0 TMA producer (Q once, then K / V^T blocks through a
-// 4-stage ring in the order the MMAs consume them); warp 1 allocates TMEM and its lane 0
-// issues the MMAs; warps 2..9 run the softmax and the epilogue, two warps per 32-row
-// band (TMEM lane quarter), each on one 64-column half of every S block: the block
-// maxima and the final sums of the two halves are combined through shared memory.  P is double-buffered so
-// that the softmax of block j + 1 overlaps the P V MMAs of block j.  V enters as V^T (a
-// K-major operand, kv contiguous, fp16), written by the QKV GEMM's epilogue or by
+// What bounds it now is shared memory: per key block of two tiles the products read 256 KB of
+// operands, P is written (64 KB) and the block arrives (64 KB), 3072 cycles at 128 bytes a cycle
+// against 3100 measured and 2048 of tensor time.  Before that the issue of the MMAs was the
+// bound (one thread of a diverged warp: 4450 cycles, whatever the softmax did).  Sixteen warps
+// share the softmax: two per band, each on one 64-column half of a block (64 scores a thread
+// leave room for all of them in registers).  S is free for the next block's product as soon as
+// its scores and the halves' maxima have been read.  Two tiles per CTA keep four such warps on
+// every scheduler and load each key block once for 256 rows.
+// Measured against one tile per CTA with eight softmax warps (kernel, us): 8 x 1536 positions,
+// 32 heads of 128: 430 -> 289 (1070 TFLOP/s); 4 x 1000, 28 q / 4 kv heads: 81 -> 55; 1 x 512: 9.3
+// -> 9.7; 32 query rows of each of 16 x 896 (28 / 4 heads): 55 -> 14; 32 rows of 1 x 1536: 18.9
+// -> 10.4.
+//
+// Where the units of a launch leave SMs idle the key axis is split over the S CTAs of a
+// cluster: each keeps (m, l, O) of its blocks, and after one cluster barrier every CTA
+// combines 1 / S of the rows, reading the S parts through distributed shared memory (in rank
+// order, so bit-reproducible).  Whether a launch splits, and takes four or eight bands per CTA,
+// follows from the rows that the row plan gives it (attn_cost); without the split a cluster's
+// CTAs are independent.
+//
+// Roles (576 threads): warp 0 lane 0 TMA producer (Q once, then K / V^T blocks through a ring
+// in the order the MMAs consume them); warp 1 allocates TMEM and issues the MMAs (a second
+// issuer, a warp per tile, gained nothing); warps 2..17 run the softmax and the epilogue (TMEM lane quarter = band of the tile).  V enters
+// as V^T (a K-major operand, kv contiguous, fp16), written by the QKV GEMM's epilogue or by
 // v_transpose_kernel from the q|k|v buffer.
 // Every wait is bounded (DERR_WAIT_TIMEOUT).
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
 namespace dcl {
 namespace {
 
-constexpr int AT_THREADS = 320;
-constexpr int AT_SOFTMAX = 8;  // softmax warps (2 .. 9)
-constexpr int AT_STAGES = 4;
+constexpr int AT_SOFTMAX = 8;  // softmax warps of a tile
+constexpr int AT_THREADS = 64 + 2 * 32 * AT_SOFTMAX;
+constexpr int AT_BANDS = 8;  // per CTA: two tiles of four
 constexpr int AT_BOX = 128 * 128;  // one 128-row x 128-byte swizzle box
+constexpr int AT_SMS = 152;
 
 template <int HD>
 struct AttnCfg {
-  static constexpr int KB = HD / 64;                   // 64-wide boxes along hd
-  static constexpr int Q_BYTES = 128 * HD * 2;         // Q tile [128][HD]
-  static constexpr int STAGE_BYTES = 128 * HD * 2;     // K block [128][HD] or V^T block [HD][128]
-  static constexpr int VBOX = HD * 128;                // one V^T box: [HD rows][64 kv]
-  static constexpr int P_BYTES = 2 * 2 * AT_BOX;       // 2 buffers of P (fp16), [128][128] each
+  static constexpr int KB = HD / 64;                // 64-wide boxes along hd
+  static constexpr int Q_BYTES = 128 * HD * 2;      // a tile of Q [128][HD]
+  static constexpr int STAGES = HD == 128 ? 3 : 6;
+  static constexpr int STAGE_BYTES = 128 * HD * 2;  // K block [128][HD] or V^T block [HD][128]
+  static constexpr int VBOX = HD * 128;             // one V^T box: [HD rows][64 kv]
+  static constexpr int P_BYTES = 2 * AT_BOX;        // a tile of P (fp16) [128][128]
   static constexpr int BARS = 256;
-  static constexpr int RED = 2 * 128 * 4;              // per-half row maxima / sums [2][128]
-  static constexpr size_t SMEM = 1024 + (size_t)Q_BYTES + AT_STAGES * STAGE_BYTES + P_BYTES + BARS + RED;
-  static constexpr uint32_t TMEM_COLS = 512;           // S double buffer (2 x 128) + O (HD)
+  static constexpr int DATA = 2 * Q_BYTES + STAGES * STAGE_BYTES + 2 * P_BYTES;
+  static constexpr int RED = 2 * 2 * 128 * 2;       // row maxima of the halves [tile][half][row], bf16
+  static constexpr size_t SMEM = 1024 + (size_t)DATA + BARS + RED;
+  static constexpr uint32_t TMEM_COLS = 512;        // S of two tiles (2 x 128), O of two (2 x HD)
+  // a split's parts: O rows in fp32 (padded by 16 bytes), then {m, l} of every row
+  static constexpr int O_PITCH = HD * 4 + 16;
+  static constexpr int ML = 256 * O_PITCH;
+  static_assert(ML + 256 * 8 <= DATA, "the parts take the place of the operands");
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
+
+// Units (CTAs' worth of bands) of a sequence with `rows` query rows.
+__host__ __device__ inline int attn_units(int rows, int rep, int bands) {
+  return (rep * ((rows + 31) / 32) + bands - 1) / bands;
+}
+// What `units` units of `bands` bands over nb key blocks take with the key axis split S ways, in
+// tenths of a key block of two tiles: rounds of CTAs, each its blocks (one tile takes 6/10 of
+// two), its start and end (2 blocks), and with a split the combination (2 blocks).
+__host__ __device__ inline long attn_cost(long units, int bands, int nb, int S) {
+  return (units * S + AT_SMS - 1) / AT_SMS *
+         ((nb + S - 1) / S * (bands > 4 ? 10 : 6) + (S > 1 ? 20 : 0) + 20);
+}
 
 // vt[(b*G + g)*hd + d][t] = v of token t, kv head g, component d (row pitch Tp, zero pad),
 // in fp16 (the bf16 values, held exactly).  A block moves a 64-token x 64-channel tile
@@ -76,55 +117,52 @@ __global__ void __launch_bounds__(256) v_transpose_kernel(const __nv_bfloat16* _
 template <int HD>
 __global__ void __launch_bounds__(AT_THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
-                   const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap to, int T, int H,
-                   int G, int kcol0, const int* __restrict__ seq_off, const int* __restrict__ seq_len, int* err) {
+                   const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap to,
+                   __nv_bfloat16* __restrict__ out, int B, int T, int H, int G, int kcol0,
+                   const int* __restrict__ seq_off, const int* __restrict__ seq_len, int mode, int bands, int* err) {
   using C = AttnCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - raw);
-  const uint32_t sQ = base;
-  const uint32_t sKV = sQ + C::Q_BYTES;
-  const uint32_t sP = sKV + AT_STAGES * C::STAGE_BYTES;  // per buffer: two 64-key boxes of P
-  const uint32_t bars = sP + C::P_BYTES;
+  const uint32_t sQ = base;                                // per tile: KB boxes
+  const uint32_t sKV = sQ + 2 * C::Q_BYTES;
+  const uint32_t sP = sKV + C::STAGES * C::STAGE_BYTES;    // per tile: two 64-key boxes of P
+  const uint32_t bars = base + C::DATA;
   const uint32_t q_full = bars;
-  const uint32_t kv_full0 = bars + 8;                   // + 8 s
-  const uint32_t kv_empty0 = kv_full0 + 8 * AT_STAGES;  // + 8 s
-  const uint32_t s_full0 = kv_empty0 + 8 * AT_STAGES;   // + 8 b
-  const uint32_t s_empty0 = s_full0 + 16;               // + 8 b
-  const uint32_t p_full0 = s_empty0 + 16;  // + 8 buffer
-  const uint32_t p_empty0 = p_full0 + 16;  // + 8 buffer
-  const uint32_t o_full = p_empty0 + 16;
-  const uint32_t drain = o_full + 8;
+  const uint32_t kv_full0 = bars + 8;                      // + 8 s
+  const uint32_t kv_empty0 = kv_full0 + 8 * C::STAGES;     // + 8 s
+  const uint32_t s_full0 = kv_empty0 + 8 * C::STAGES;      // + 8 tile
+  const uint32_t s_empty0 = s_full0 + 16;
+  const uint32_t p_full0 = s_empty0 + 16;
+  const uint32_t p_empty0 = p_full0 + 16;
+  const uint32_t drain = p_empty0 + 16;
   const uint32_t holder = drain + 8;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
-  float* red = reinterpret_cast<float*>(smem + (bars + C::BARS - base));  // [2][128]
+  __nv_bfloat16* red = reinterpret_cast<__nv_bfloat16*>(smem + C::DATA + C::BARS);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // grid (head, sequence, query tile): the query tile is the slowest index, so that the
-  // CTAs with work come first in dispatch order
-  const int h = blockIdx.x, b = blockIdx.y, qt = blockIdx.z;
-  const int g = h / (H / G);
-  const int nb = (T + 127) / 128;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
+  const int S = (int)cluster_size(), rank = (int)cluster_rank();
+  // grid (rank, kv head, unit-major sequence): the unit is the slowest index, so that the CTAs
+  // with work come first in dispatch order
+  const int g = blockIdx.y, b = blockIdx.z % B, zc = blockIdx.z / B;
+  const int rep = H / G, nb = (T + 127) / 128;
 
   // set-up first (it reads nothing that earlier kernels write), so that under programmatic
   // dependent launch it overlaps the tail of the kernel before
   if (threadIdx.x == 0) {
     mbar_init(q_full, 1);
-    for (int s = 0; s < AT_STAGES; ++s) {
+    for (int s = 0; s < C::STAGES; ++s) {
       mbar_init(kv_full0 + 8 * s, 1);
       mbar_init(kv_empty0 + 8 * s, 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(s_full0 + 8 * i, 1);
-      mbar_init(s_empty0 + 8 * i, AT_SOFTMAX);  // the softmax warps
-    }
-    for (int i = 0; i < 2; ++i) {
+      mbar_init(s_empty0 + 8 * i, AT_SOFTMAX);  // the tile's softmax warps
       mbar_init(p_full0 + 8 * i, AT_SOFTMAX);
       mbar_init(p_empty0 + 8 * i, 1);
     }
-    mbar_init(o_full, 1);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -141,14 +179,39 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
 
   pdl_wait();  // the previous kernels of the step (the row plan among them) have completed
   pdl_launch_dependents();
-  // the query rows of sequence b are rows [off, off + len) of q and of the output; a tile
-  // past them has nothing to do and leaves at once (uniform over the CTA)
+  // the query rows of sequence b are rows [off, off + len) of q and of the output
   const int q_off = seq_off ? seq_off[b] : b * T;
   const int q_len = seq_len ? seq_len[b] : T;
-  if (qt * 128 >= q_len) {
+  bool split = mode == ATTN_SPLIT;
+  if (mode == ATTN_BY_ROWS) {
+    // the cheapest of whole or split units of eight or four bands that the grid has CTAs for
+    int total[2] = {0, 0}, most[2] = {0, 0};  // of eight, of four
+    for (int i = lane; i < B; i += 32)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int n = attn_units(seq_len[i], rep, 8 >> k);
+        total[k] += n;
+        most[k] = max(most[k], n);
+      }
+    const int Z = gridDim.z / B;
+    long best = 0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int n = (int)__reduce_add_sync(0xffffffffu, (unsigned)total[k]) * G;
+      const int mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)most[k]);
+      const long whole = attn_cost(n, 8 >> k, nb, 1), parts = attn_cost(n, 8 >> k, nb, S);
+      if (k == 0 || (mx <= Z * S && whole < best)) best = whole, bands = 8 >> k, split = false;
+      if (mx <= Z && S > 1 && parts < best) best = parts, bands = 8 >> k, split = true;
+    }
+  }
+  const int nch = (q_len + 31) / 32, nbands = rep * nch;  // band i: head i / nch, rows 32 (i % nch) ..
+  const int band0 = (split ? zc : zc * S + rank) * bands;
+  if (band0 >= nbands) {  // nothing to do (all CTAs of the cluster, if split): uniform over the CTA
     if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
     return;
   }
+  const int live = min(bands, nbands - band0), ntiles = (live + 3) / 4;
+  const int jb = split ? rank * nb / S : 0, n = (split ? (rank + 1) * nb / S : nb) - jb;  // its key blocks
 
   if (warp == 0) {
     if (lane == 0) {
@@ -157,26 +220,16 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
       int stage = 0;
       uint32_t phase = 0;
       long issued = 0;
-      mbar_arrive_expect_tx(q_full, C::Q_BYTES);
-      for (int bx = 0; bx < C::KB; ++bx) tma_load_2d(sQ + bx * AT_BOX, &tq, h * HD + bx * 64, q_off + qt * 128, q_full);
-      // consumption order: K_0, K_1, then per j: K_{j+2}, V_j (K only while j + 2 < nb)
-      const int n_loads = 2 * nb;
-      const int head = nb < 2 ? nb : 2, npairs = nb > 2 ? nb - 2 : 0;
-      for (int u = 0; u < n_loads && ok; ++u) {
-        bool is_v;
-        int j;
-        if (u < head) {
-          is_v = false, j = u;
-        } else {
-          const int r = u - head;
-          if (r < 2 * npairs) {
-            is_v = (r & 1) != 0;
-            j = (r >> 1) + (is_v ? 0 : 2);
-          } else {
-            is_v = true;
-            j = npairs + (r - 2 * npairs);
-          }
-        }
+      mbar_arrive_expect_tx(q_full, live * 32 * HD * 2);
+      for (int i = 0; i < live; ++i) {
+        const int h = g * rep + (band0 + i) / nch, r0 = q_off + 32 * ((band0 + i) % nch);
+        const uint32_t dst = sQ + (i >> 2) * C::Q_BYTES + (i & 3) * (32 * 128);
+        for (int bx = 0; bx < C::KB; ++bx) tma_load_2d(dst + bx * AT_BOX, &tq, h * HD + bx * 64, r0, q_full);
+      }
+      // consumption order: K_0, then per block K_{j+1}, V_j
+      for (int u = 0; u < 2 * n; ++u) {
+        const bool is_v = u == 2 * n - 1 || (u > 0 && (u & 1) == 0);
+        const int j = jb + (is_v ? (u - 1) >> 1 : (u + 1) >> 1);
         if (!mbar_wait(kv_empty0 + 8 * stage, phase ^ 1u, abort_flag)) {
           ok = false;
           break;
@@ -190,7 +243,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
           for (int bx = 0; bx < 2; ++bx) tma_load_3d(dst + bx * C::VBOX, &tv, j * 128 + bx * 64, 0, b * G + g, bar);
         }
         ++issued;
-        if (++stage == AT_STAGES) {
+        if (++stage == C::STAGES) {
           stage = 0;
           phase ^= 1u;
         }
@@ -201,229 +254,241 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         // wait (bounded) for the copies this thread issued before leaving
         volatile int no_abort = 0;
         mbar_wait(q_full, 0, &no_abort);
-        for (int s = 0; s < AT_STAGES && s < issued; ++s) {
-          const long arms = (issued - 1 - s) / AT_STAGES + 1;
+        for (int s = 0; s < C::STAGES && s < issued; ++s) {
+          const long arms = (issued - 1 - s) / C::STAGES + 1;
           mbar_wait(kv_full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------ MMA issuer
-      constexpr uint32_t idesc_s = make_idesc(128, 128);
-      constexpr uint32_t idesc_o = make_idesc_f16(128, HD);  // fp16 P and V
-      bool ok = mbar_wait(q_full, 0, abort_flag);
-      int stage = 0;
-      uint32_t phase = 0;
-      int si = 0;  // S-buffer uses so far
-      auto take = [&](uint32_t& st_addr) -> bool {
-        if (!mbar_wait(kv_full0 + 8 * stage, phase, abort_flag)) return false;
-        st_addr = sKV + stage * C::STAGE_BYTES;
-        return true;
-      };
-      auto release = [&]() {
-        umma_commit(kv_empty0 + 8 * stage);
-        if (++stage == AT_STAGES) {
-          stage = 0;
-          phase ^= 1u;
+    // ------------------------------------------------ MMA issuer (the whole warp, one lane issues)
+    constexpr uint32_t idesc_s = make_idesc(128, 128);
+    constexpr uint32_t idesc_o = make_idesc_f16(128, HD);  // fp16 P and V
+    const bool leader = elect_one();
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      return (bool)__all_sync(0xffffffffu, mbar_wait_inline(bar, parity, abort_flag));
+    };
+    bool ok = wait(q_full, 0);
+    int stage = 0;
+    uint32_t phase = 0;
+    auto next_stage = [&]() {
+      if (++stage == C::STAGES) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    };
+    auto issue_s = [&](int j) -> bool {  // S = Q K_j^T of both tiles
+      if (!wait(kv_full0 + 8 * stage, phase)) return false;
+      const uint64_t dk = sw128_desc(sKV + stage * C::STAGE_BYTES);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (t >= ntiles) break;
+        if (!wait(s_empty0 + 8 * t, ((uint32_t)j & 1u) ^ 1u)) return false;
+        tc_fence_after();
+        const uint64_t dq = sw128_desc(sQ + t * C::Q_BYTES);
+        if (leader) {
+#pragma unroll
+          for (int k = 0; k < HD / 16; ++k)
+            umma_bf16(tmem + 128u * t, dq + (k >> 2) * (AT_BOX >> 4) + 2 * (k & 3), dk + (k >> 2) * (AT_BOX >> 4) + 2 * (k & 3),
+                      idesc_s, k > 0 ? 1u : 0u);
+          umma_commit(s_full0 + 8 * t);
+          if (t + 1 == ntiles) umma_commit(kv_empty0 + 8 * stage);
         }
-      };
-      auto issue_s = [&]() -> bool {  // S[si & 1] = Q K^T with the K block at the ring head
-        uint32_t kaddr;
-        if (!take(kaddr)) return false;
-        const int sb = si & 1;
-        if (!mbar_wait(s_empty0 + 8 * sb, (((uint32_t)si >> 1) & 1u) ^ 1u, abort_flag)) return false;
-        tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)(sb * 128);
-#pragma unroll
-        for (int k = 0; k < HD / 16; ++k)
-          umma_bf16(d, sw128_desc(sQ + (k >> 2) * AT_BOX) + 2 * (k & 3), sw128_desc(kaddr + (k >> 2) * AT_BOX) + 2 * (k & 3),
-                    idesc_s, k > 0 ? 1u : 0u);
-        release();
-        umma_commit(s_full0 + 8 * sb);
-        ++si;
-        return true;
-      };
-      auto issue_pv = [&](int j) -> bool {  // O += P_j V_j (fp16 operands)
-        uint32_t vaddr;
-        if (!take(vaddr)) return false;
-        const int pb = j & 1;
-        if (!mbar_wait(p_full0 + 8 * pb, ((uint32_t)j >> 1) & 1u, abort_flag)) return false;
-        tc_fence_after();
-        const uint32_t d = tmem + 256u;
-        const uint32_t pbase = sP + (uint32_t)pb * 2 * AT_BOX;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          umma_bf16(d, sw128_desc(pbase + (k >> 2) * AT_BOX) + 2 * (k & 3), sw128_desc(vaddr + (k >> 2) * C::VBOX) + 2 * (k & 3),
-                    idesc_o, (j > 0 || k > 0) ? 1u : 0u);
-        release();
-        umma_commit(p_empty0 + 8 * pb);
-        return true;
-      };
-      if (ok) ok = issue_s();  // S_0, S_1
-      if (ok && nb > 1) ok = issue_s();
-      for (int j = 0; ok && j < nb; ++j) {  // S_{j+2} (its buffer frees with P_j) before PV_j
-        if (j + 2 < nb) ok = issue_s();
-        if (ok) ok = issue_pv(j);
+        __syncwarp();
       }
-      if (ok) umma_commit(o_full);
-      if (!ok) {
-        *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
+      next_stage();
+      return true;
+    };
+    auto issue_pv = [&](int j) -> bool {  // O += P_j V_j of both tiles (fp16 operands)
+      if (!wait(kv_full0 + 8 * stage, phase)) return false;
+      const uint64_t dv = sw128_desc(sKV + stage * C::STAGE_BYTES);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (t >= ntiles) break;
+        if (!wait(p_full0 + 8 * t, (uint32_t)j & 1u)) return false;
+        tc_fence_after();
+        const uint64_t dp = sw128_desc(sP + t * C::P_BYTES);
+        if (leader) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            umma_bf16(tmem + 256u + (uint32_t)(HD * t), dp + (k >> 2) * (AT_BOX >> 4) + 2 * (k & 3),
+                      dv + (k >> 2) * (C::VBOX >> 4) + 2 * (k & 3), idesc_o, (j > 0 || k > 0) ? 1u : 0u);
+          umma_commit(p_empty0 + 8 * t);
+          if (t + 1 == ntiles) umma_commit(kv_empty0 + 8 * stage);
+        }
+        __syncwarp();
       }
-      umma_commit(drain);  // every MMA issued here completes before TMEM is released
-      volatile int no_abort = 0;
-      mbar_wait(drain, 0, &no_abort);
+      next_stage();
+      return true;
+    };
+    if (ok) ok = issue_s(0);
+    for (int j = 0; ok && j < n; ++j) {  // S_{j+1} (its buffer frees early in the softmax of j) before P V of j
+      if (j + 1 < n) ok = issue_s(j + 1);
+      if (ok) ok = issue_pv(j);
     }
+    if (!ok) {
+      *abort_flag = 1;
+      if (leader) report_error(err, DERR_WAIT_TIMEOUT);
+    }
+    if (leader) umma_commit(drain);  // every MMA issued here completes before TMEM is released
+    __syncwarp();
+    volatile int no_abort = 0;
+    mbar_wait(drain, 0, &no_abort);
   } else {
-    // ------------------------------------------------ softmax + epilogue (warps 2..9)
-    const int q = warp & 3;             // TMEM lane quarter = 32-row band
-    const int hs = (warp - 2) >> 2;     // which 64-column half of each S block
-    const int co = 64 * hs;
-    const int r = q * 32 + lane;        // query row within the tile
+    // ------------------------------------------------ softmax + epilogue (warps 2..17)
+    const int w = warp - 2, tile = w / AT_SOFTMAX, hs = (w >> 2) & 1;  // hs: which 64 columns of a block
+    const int q = warp & 3;                                            // TMEM lane quarter = band of the tile
+    const int r = q * 32 + lane;                                       // query row within the tile
+    const bool work = 4 * tile + q < live;
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    auto softmax_bar = []() { asm volatile("bar.sync 1, %0;" ::"n"(AT_SOFTMAX * 32) : "memory"); };
+    const uint32_t ts = tmem + lane_off + 128u * tile + 64u * hs;
+    const uint32_t to_col = tmem + lane_off + 256u + (uint32_t)(HD * tile);
+    const uint32_t sPt = sP + tile * C::P_BYTES;
+    const uint32_t s_full = s_full0 + 8 * tile, s_empty = s_empty0 + 8 * tile, p_full = p_full0 + 8 * tile,
+                   p_empty = p_empty0 + 8 * tile;
+    __nv_bfloat16* mine = red + (tile * 2 + hs) * 128 + r;
+    const __nv_bfloat16* other = red + (tile * 2 + (hs ^ 1)) * 128 + r;
+    auto band_bar = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1u + 4u * tile + q) : "memory"); };  // the band's two warps
+    constexpr int OH = HD / 2;  // O columns of this warp: [hs * OH, + OH)
     const float scale2 = kLog2e * rsqrtf((float)HD);
-    // One pass over the key blocks with a running maximum.  Per block: this half's 64
-    // columns of S from TMEM, the block's row maximum combined with the partner warp's
-    // half through shared memory, then P = exp2(S scale - m) against the running maximum
-    // m.  m is raised only when a block's maximum exceeds it by more than 8 (so P <= 2^8,
-    // exact in fp32 and in the hi / lo split); l and this warp's half of O are then scaled
-    // by 2^(m_old - m_new) once the previous P V product has completed.  O and l carry
-    // the same factor, so O / l is the softmax of the exact-maximum form.
     bool ok = true;
     float m = -INFINITY, l = 0.f;
-    const uint32_t band_bar_id = 2u + (uint32_t)q;  // the two warps of this 32-row band
-    auto band_bar = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(band_bar_id) : "memory"); };
-    for (int j = 0; j < nb; ++j) {  // (no early exit: both warps of a band meet at every barrier)
-      const int sb = j & 1, pb = j & 1;
-      if (ok) ok = mbar_wait(s_full0 + 8 * sb, ((uint32_t)j >> 1) & 1u, abort_flag);
-      if (ok && j >= 2) ok = mbar_wait(p_empty0 + 8 * pb, ((uint32_t)(j - 2) >> 1) & 1u, abort_flag);  // PV_{j-2} read it
-      ok = __all_sync(0xffffffffu, ok);
-      const int valid = T - j * 128 - co;  // live columns of this half
+    for (int j = 0; tile < ntiles && j < n; ++j) {  // (no early exit: both warps of a band meet at every barrier)
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait_inline(s_full, (uint32_t)j & 1u, abort_flag));
       uint32_t v[2][32];
-      float mm = -INFINITY;
-      if (ok) {
-        tc_fence_after();
+      float f = 1.f;
+      bool rescale = false;
+      if (work) {
+        float mm = -INFINITY;
+        if (ok) {
+          tc_fence_after();
 #pragma unroll
-        for (int c = 0; c < 2; ++c) tmem_ld32(tmem + lane_off + (uint32_t)(sb * 128 + co + 32 * c), v[c]);
-        tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(s_empty0 + 8 * sb);  // the S buffer is free for S_{j+2}
-        if (valid >= 64) {
+          for (int c = 0; c < 2; ++c) tmem_ld32(ts + 32u * c, v[c]);
+          tmem_ld_wait();
+          tc_fence_before();
+          const int valid = T - (jb + j) * 128 - 64 * hs;  // live columns of the half block
+          if (valid < 64) {
+            asm volatile("" ::: "memory");  // (a branch: not 64 selects in every block)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+              for (int e = 0; e < 32; ++e)
+                if (32 * c + e >= valid) v[c][e] = __float_as_uint(-INFINITY);
+          }
           // four independent three-input maximum chains over the 64 columns
-          float a4[4];
+          float mx[4];
 #pragma unroll
           for (int t = 0; t < 4; ++t) {
-            const uint32_t* w = &v[t >> 1][(t & 1) * 16];
-            float acc = f32(w[0]);
+            const uint32_t* vw = &v[t >> 1][(t & 1) * 16];
+            float acc = f32(vw[0]);
 #pragma unroll
-            for (int e = 1; e < 15; e += 2) acc = max3f(acc, f32(w[e]), f32(w[e + 1]));
-            a4[t] = fmaxf(acc, f32(w[15]));
+            for (int e = 1; e < 15; e += 2) acc = max3f(acc, f32(vw[e]), f32(vw[e + 1]));
+            mx[t] = fmaxf(acc, f32(vw[15]));
           }
-          mm = max3f(a4[0], a4[1], fmaxf(a4[2], a4[3]));
-        } else {
-#pragma unroll
-          for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int e = 0; e < 32; ++e)
-              if (32 * c + e < valid) mm = fmaxf(mm, f32(v[c][e]));
+          mm = max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])) * scale2;
         }
+        // the halves agree on a maximum; its bf16 rounding serves (any m that both use will do,
+        // and P stays below 2^9)
+        const __nv_bfloat16 own = __float2bfloat16_rn(mm);
+        *mine = own;
+        band_bar();
+        const float mb = fmaxf(__bfloat162float(own), __bfloat162float(*other));
+        __syncwarp();
+        if (lane == 0 && ok) mbar_arrive(s_empty);  // scores and maxima read: the next block's may be written
+        if (ok) {
+          const bool raise = mb > m + 8.f;  // always at the first block (m = -inf)
+          rescale = j > 0 && __any_sync(0xffffffffu, raise);
+          if (raise) {
+            f = ex2_approx(m - mb);
+            m = mb;
+          }
+        }
+      } else if (lane == 0 && ok) {
+        mbar_arrive(s_empty);
       }
-      red[hs * 128 + r] = mm * scale2;
-      band_bar();
-      const float mb = fmaxf(red[r], red[128 + r]);
-      band_bar();  // both halves read before the next block writes the slots
+      // P V of the block before has read this tile's P (and its O is complete)
+      if (ok && j > 0) ok = __all_sync(0xffffffffu, mbar_wait_inline(p_empty, (uint32_t)(j - 1) & 1u, abort_flag));
       if (!ok) continue;
-      const bool raise = mb > m + 8.f;  // always at the first block (m = -inf)
-      if (j > 0 && __any_sync(0xffffffffu, raise)) {
-        // rescale l and this warp's O columns; P V_{j-1} must have completed first
-        if (!mbar_wait(p_empty0 + 8 * ((j - 1) & 1), ((uint32_t)(j - 1) >> 1) & 1u, abort_flag)) ok = false;
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) continue;
+      if (rescale) {  // warp-uniform, rare: in small pieces beside the scores
         tc_fence_after();
-        const float f = raise ? ex2_approx(m - mb) : 1.f;
 #pragma unroll 1
-        for (int c = co; c < HD && c < co + 64; c += 32) {
-          uint32_t ov[32];
-          tmem_ld32(tmem + lane_off + 256u + (uint32_t)c, ov);
+        for (int c = hs * OH; c < (hs + 1) * OH; c += 8) {
+          uint32_t ov[8];
+          tmem_ld8(to_col + (uint32_t)c, ov);
           tmem_ld_wait();
-          float o[32];
 #pragma unroll
-          for (int e = 0; e < 32; ++e) o[e] = f32(ov[e]) * f;
-          tmem_st32(tmem + lane_off + 256u + (uint32_t)c, o);
+          for (int e = 0; e < 8; ++e) ov[e] = __float_as_uint(f32(ov[e]) * f);
+          tmem_st8(to_col + (uint32_t)c, ov);
         }
         tmem_st_wait();
         tc_fence_before();
-        l *= f;
       }
-      if (raise) m = mb;
-      const uint32_t box = sP + (uint32_t)pb * 2 * AT_BOX + (uint32_t)hs * AT_BOX;
-      const bool full = valid >= 64;
-      // the block's sum of this half, in two packed partial sums (fixed order)
-      unsigned long long la = 0ull, lb = 0ull;
-      const unsigned long long sc2 = pk2(scale2, scale2), nm2 = pk2(-m, -m);
+      if (work) {
+        // the half block's sum in four packed partial sums (fixed order)
+        unsigned long long ls[4] = {0ull, 0ull, 0ull, 0ull};
+        const unsigned long long sc2 = pk2(scale2, scale2), nm2 = pk2(-m, -m);
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        // P in fp16 (round to nearest even: 2^-12 relative, P <= 2^8); l sums the fp32 values
-        float pv[32];
-        if (full) {  // the exponent arguments two lanes per instruction, no column mask
+        for (int k = 0; k < 8; ++k) {
+          uint32_t pk[4];
 #pragma unroll
-          for (int e = 0; e < 32; e += 2) {
+          for (int e = 0; e < 4; ++e) {
+            const int i = 8 * (k & 3) + 2 * e;
             float y0, y1;
-            upk2(ffma2(pk2(f32(v[c][e]), f32(v[c][e + 1])), sc2, nm2), y0, y1);
-            pv[e] = ex2_approx(y0);
-            pv[e + 1] = ex2_approx(y1);
+            upk2(ffma2(pk2(f32(v[k >> 2][i]), f32(v[k >> 2][i + 1])), sc2, nm2), y0, y1);
+            const float p0 = ex2_approx(y0), p1 = ex2_approx(y1);
+            ls[e] = fadd2(ls[e], pk2(p0, p1));
+            pk[e] = pack_f16x2(p0, p1);  // round to nearest even: 2^-12 relative
           }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            pv[e] = ex2_approx(fmaf(f32(v[c][e]), scale2, -m));
-            if (32 * c + e >= valid) pv[e] = 0.f;
-          }
+          st_shared_v4(sPt + (uint32_t)hs * AT_BOX + swz(r, k), pk[0], pk[1], pk[2], pk[3]);
         }
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          la = fadd2(la, pk2(pv[e], pv[e + 1]));
-          lb = fadd2(lb, pk2(pv[e + 2], pv[e + 3]));
-        }
-        const int k0 = c * 4;
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          st_shared_v4(box + swz(r, k0 + k), pack_f16x2(pv[8 * k], pv[8 * k + 1]), pack_f16x2(pv[8 * k + 2], pv[8 * k + 3]),
-                       pack_f16x2(pv[8 * k + 4], pv[8 * k + 5]), pack_f16x2(pv[8 * k + 6], pv[8 * k + 7]));
+        float a0, a1;
+        upk2(fadd2(fadd2(ls[0], ls[1]), fadd2(ls[2], ls[3])), a0, a1);
+        l = l * (j > 0 ? f : 1.f) + (a0 + a1);
+        tc_fence_before();
+        fence_proxy_async_smem();  // P is read by the tensor cores (async proxy)
       }
-      {
-        float a0, a1, b0, b1;
-        upk2(la, a0, a1);
-        upk2(lb, b0, b1);
-        l += (a0 + b0) + (a1 + b1);
-      }
-      tc_fence_before();
-      fence_proxy_async_smem();  // P is read by the tensor cores (async proxy)
       __syncwarp();
-      if (lane == 0) mbar_arrive(p_full0 + 8 * pb);
+      if (lane == 0) mbar_arrive(p_full);
     }
-    // the row sum over both halves, half 0 + half 1 (a fixed order)
-    red[hs * 128 + r] = l;
-    softmax_bar();
-    l = red[r] + red[128 + r];
-    if (ok) ok = mbar_wait(o_full, 0, abort_flag);
-    ok = __all_sync(0xffffffffu, ok);
-    if (ok) {
-      // epilogue: O / l -> bf16 -> TMA store, each warp one 64-column box of its band
-      // (staged in the P buffers, free once every PV MMA has completed)
-      tc_fence_after();
-      const float inv = 1.0f / l;
-      const int row0 = qt * 128 + q * 32;
+    if (ok && tile < ntiles) ok = __all_sync(0xffffffffu, mbar_wait_inline(p_empty, (uint32_t)(n - 1) & 1u, abort_flag));
+    tc_fence_after();
+    if (work) {  // the row sum, half 0 + half 1 (through the tile's Q, which every product has read)
+      float* sums = reinterpret_cast<float*>(smem + (sQ - base) + tile * C::Q_BYTES);
+      if (ok) sums[hs * 128 + r] = l;
+      band_bar();
+      if (ok) l = sums[r] + sums[128 + r];
+    }
+    if (split) {
+      // every tile's operands are done with: this CTA's part takes their place
+      asm volatile("bar.sync 9, %0;" ::"n"(64 * AT_SOFTMAX) : "memory");
+      if (ok && work) {
+        const uint32_t row = (uint32_t)(128 * tile + r), at = base + row * C::O_PITCH;
 #pragma unroll 1
-      for (int c = co; c < HD; c += 128) {
-        const uint32_t bx = sP + (uint32_t)((q * 2 + hs) * (32 * 128));
+        for (int c = hs * OH; c < (hs + 1) * OH; c += 32) {
+          uint32_t v[32];
+          tmem_ld32(to_col + (uint32_t)c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            st_shared_v4(at + (uint32_t)(c * 4 + 16 * k), v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+        }
+        if (hs == 0) {
+          st_shared_f32(base + C::ML + 8 * row, m);
+          st_shared_f32(base + C::ML + 8 * row + 4, l);
+        }
+      }
+    } else if (ok && work) {
+      // epilogue: O / l -> bf16 -> TMA store, each warp one 64-column box of its band (staged in
+      // the tile's P, free once every P V MMA has completed)
+      const float inv = 1.0f / l;
+      const int band = band0 + 4 * tile + q, row0 = 32 * (band % nch), col0 = (g * rep + band / nch) * HD;
+#pragma unroll 1
+      for (int c = 64 * hs; c < HD; c += 128) {
+        const uint32_t bx = sPt + (uint32_t)((q * C::KB + (c >> 6)) * (32 * 128));
 #pragma unroll 1
         for (int hh = 0; hh < 2; ++hh) {
           uint32_t v[32];
-          tmem_ld32(tmem + lane_off + 256u + (uint32_t)(c + 32 * hh), v);
+          tmem_ld32(to_col + (uint32_t)(c + 32 * hh), v);
           tmem_ld_wait();
           float o[32];
 #pragma unroll
@@ -435,11 +500,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         }
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0 && row0 < q_len) {
+        if (lane == 0) {
           if (seq_off)
-            tma_store_2d(&to, bx, h * HD + c, q_off + row0);
+            tma_store_2d(&to, bx, col0 + c, q_off + row0);
           else
-            tma_store_3d(&to, bx, h * HD + c, row0, b);
+            tma_store_3d(&to, bx, col0 + c, row0, b);
         }
       }
       if (lane == 0) {
@@ -457,13 +522,89 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    __syncwarp();
     tc_fence_after();
     tmem_dealloc(tmem, C::TMEM_COLS);
   }
+  if (split) {
+    __syncwarp();
+    cluster_sync();  // every CTA of the cluster has its part in shared memory
+    if (warp >= 2 && !*abort_flag) {
+      // this CTA's share of the rows, four columns a thread
+      const int rows = 32 * live, i1 = (rank + 1) * rows / S * (HD / 4);
+      for (int i = rank * rows / S * (HD / 4) + (int)threadIdx.x - 64; i < i1; i += 64 * AT_SOFTMAX) {
+        const int row = i / (HD / 4), c = 4 * (i % (HD / 4));
+        const int band = band0 + (row >> 5), t = 32 * (band % nch) + (row & 31);
+        float mx = -INFINITY, ms[8], ls[8];
+        float4 o[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+          if (s < S) {
+            const uint32_t from = map_cluster(base, s);
+            const float2 ml = ld_cluster_v2(from + C::ML + 8 * row);
+            o[s] = ld_cluster_v4(from + row * C::O_PITCH + 4 * c);
+            ms[s] = ml.x;
+            ls[s] = ml.y;
+            mx = fmaxf(mx, ml.x);
+          }
+        float l = 0.f;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < 8; ++s)
+          if (s < S) {
+            const float f = ex2_approx(ms[s] - mx);
+            l += ls[s] * f;
+            a.x += o[s].x * f;
+            a.y += o[s].y * f;
+            a.z += o[s].z * f;
+            a.w += o[s].w * f;
+          }
+        if (t < q_len) {
+          const float inv = 1.0f / l;
+          *reinterpret_cast<uint2*>(out + (size_t)(q_off + t) * H * HD + (g * rep + band / nch) * HD + c) =
+              make_uint2(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(a.z * inv, a.w * inv));
+        }
+      }
+    }
+    __syncwarp();
+    cluster_sync_relaxed();  // no CTA leaves while another may read its part
+  }
+}
+
+// The launch's cluster size, clusters per (sequence, kv head), bands per CTA and whether the
+// kernel decides on the last and on the split.
+struct AttnShape {
+  int S, Z, bands, mode;
+};
+
+AttnShape attn_shape(const AttnPlan& p, const AttnRows& r) {
+  const int nb = (p.T + 127) / 128, rep = p.H / p.G;
+  AttnShape a{1, 0, 8, ATTN_WHOLE};
+  if (r.exact) {  // every sequence has r.most rows: the cheapest choice, made here
+    long best = 0;
+    for (int bands = 8; bands >= 4; bands -= 4) {
+      const int units = attn_units(r.most, rep, bands);
+      for (int S = 1; S <= 8 && S <= nb; S *= 2) {
+        const long c = attn_cost((long)p.G * p.batch * units, bands, nb, S);
+        if (!a.Z || c < best) best = c, a = {S, units, bands, S > 1 ? ATTN_SPLIT : ATTN_WHOLE};
+      }
+    }
+    return a;
+  }
+  // the rows are the row plan's.  Clusters as far as the few rows of `r.seqs` sequences leave
+  // SMs idle, of two CTAs where a launch may hold many rows; CTAs for the most rows in units of
+  // eight bands, and where few units fit the GPU for smaller or split ones.
+  const int units = attn_units(r.most, rep, 8);
+  const long U = (long)p.G * r.seqs * attn_units(std::min(r.most, (r.total + r.seqs - 1) / r.seqs), rep, 8);
+  while (a.S < 8 && 2 * a.S <= nb && U * 2 * a.S <= AT_SMS) a.S *= 2;
+  if (a.S == 1 && nb >= 4) a.S = 2;
+  a.mode = ATTN_BY_ROWS;
+  a.Z = std::max((units + a.S - 1) / a.S, std::min(attn_units(r.most, rep, 4), std::max(1, 192 / (p.G * r.seqs))));
+  return a;
 }
 
 template <int HD>
-cudaError_t launch_attn(const AttnPlan& p, int* err, cudaStream_t stream) {
+cudaError_t launch_attn(const AttnPlan& p, const AttnRows& rows, int* err, cudaStream_t stream) {
   static bool attr_set = false;
   auto kern = attn_tc_kernel<HD>;
   if (!attr_set) {
@@ -471,9 +612,23 @@ cudaError_t launch_attn(const AttnPlan& p, int* err, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  dim3 grid(p.H, p.batch, (p.T + 127) / 128);
-  return launch_pdl(kern, grid, AT_THREADS, AttnCfg<HD>::SMEM, stream, p.tq, p.tk, p.tv, p.to, p.T, p.H, p.G, p.kcol0,
-                    p.seq_off, p.seq_len, err);
+  const AttnShape a = attn_shape(p, rows);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.S, p.G, a.Z * p.batch);
+  cfg.blockDim = dim3(AT_THREADS);
+  cfg.dynamicSmemBytes = AttnCfg<HD>::SMEM;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = a.S;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, p.tq, p.tk, p.tv, p.to, p.out, p.batch, p.T, p.H, p.G, p.kcol0, p.seq_off,
+                            p.seq_len, a.mode, a.bands, err);
 }
 
 }  // namespace
@@ -489,10 +644,10 @@ cudaError_t attention_plan(AttnPlan* p, const __nv_bfloat16* qkv, const __nv_bfl
       (reinterpret_cast<uintptr_t>(out) & 15) || (kbuf && (reinterpret_cast<uintptr_t>(kbuf) & 15)))
     return cudaErrorInvalidValue;
   const uint64_t cols = (uint64_t)(H + 2 * G) * hd, ocols = (uint64_t)H * hd, Tp = attn_vt_pitch(T);
-  {  // q rows of the step: [rows_max][cols]
+  {  // q rows of the step, a band at a time: [rows_max][cols]
     const uint64_t dims[2] = {cols, (uint64_t)rows_max};
     const uint64_t strides[1] = {cols * 2};
-    const uint32_t box[2] = {64, 128};
+    const uint32_t box[2] = {64, 32};
     if (!encode_tmap(&p->tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16*>(qkv), dims, strides, box,
                      CU_TENSOR_MAP_SWIZZLE_128B))
       return cudaErrorInvalidValue;
@@ -528,6 +683,7 @@ cudaError_t attention_plan(AttnPlan* p, const __nv_bfloat16* qkv, const __nv_bfl
       return cudaErrorInvalidValue;
   }
   p->qkv = qkv;
+  p->out = out;
   p->vt = vt;
   p->seq_off = seq_off;
   p->seq_len = seq_len;
@@ -546,13 +702,13 @@ cudaError_t attention_transpose_launch(const AttnPlan& p, cudaStream_t stream) {
                     (p.H + p.G) * p.hd, ghd);
 }
 
-cudaError_t attention_core_launch(const AttnPlan& p, int* err, cudaStream_t stream) {
-  return p.hd == 128 ? launch_attn<128>(p, err, stream) : launch_attn<64>(p, err, stream);
+cudaError_t attention_core_launch(const AttnPlan& p, const AttnRows& rows, int* err, cudaStream_t stream) {
+  return p.hd == 128 ? launch_attn<128>(p, rows, err, stream) : launch_attn<64>(p, rows, err, stream);
 }
 
-cudaError_t attention_launch(const AttnPlan& p, int* err, cudaStream_t stream) {
+cudaError_t attention_launch(const AttnPlan& p, const AttnRows& rows, int* err, cudaStream_t stream) {
   const cudaError_t e = attention_transpose_launch(p, stream);
-  return e != cudaSuccess ? e : attention_core_launch(p, err, stream);
+  return e != cudaSuccess ? e : attention_core_launch(p, rows, err, stream);
 }
 
 }  // namespace dcl

@@ -239,6 +239,11 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
   const int d = m.d_model;
   const std::vector<FewPlan>* few = branch == STEP_PAIR ? nullptr : &c->few[branch == STEP_FEW32 ? 0 : 1];
   const int rows = std::min(R, branch == STEP_FEW32 ? 32 : branch == STEP_FEW ? FEW_MAX_ROWS : R);  // at most
+  AttnRows ar;  // the attention's query rows: every position, or as the row plan says
+  ar.most = std::min(c->T, rows);
+  ar.total = rows;
+  ar.seqs = c->kv_fused ? std::min(c->B, std::max(1, rows / 32)) : c->B;
+  ar.exact = !c->kv_fused;
   if (h_in) {
     if (q.err == cudaSuccess)
       q.err = cudaMemcpyAsync(c->h, h_in, sizeof(float) * R * d, cudaMemcpyDeviceToDevice, c->stream);
@@ -267,7 +272,7 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
       q.end(attention_transpose_launch(c->attn_plans[l], c->stream), "v_transpose");
     }
     q.begin(DCL_K_ATTENTION);
-    q.end(attention_core_launch(c->attn_plans[l], c->derr, c->stream), "attention");
+    q.end(attention_core_launch(c->attn_plans[l], ar, c->derr, c->stream), "attention");
     q.begin(DCL_K_GEMM_O);
     q.end(F ? few_launch(F[1], c->derr, c->stream) : gemm_launch(P[1], c->derr, c->stream), "gemm_o");
     q.begin(DCL_K_RMSNORM);
@@ -1320,7 +1325,12 @@ dcl_status dcl_op_attention(dcl_ctx* c, const void* qkv_dev, void* out_dev, int3
     release();
     return fail(c, DCL_ERR_INVALID_ARG, "attention: operands must be 16-byte aligned");
   }
-  const cudaError_t e = attention_launch(pl, c->derr, c->stream);
+  AttnRows ar;
+  ar.most = q_rows ? q_rows : T;
+  ar.total = batch * ar.most;
+  ar.seqs = batch;
+  ar.exact = true;
+  const cudaError_t e = attention_launch(pl, ar, c->derr, c->stream);
   if (e != cudaSuccess) {
     release();
     return fail(c, DCL_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
