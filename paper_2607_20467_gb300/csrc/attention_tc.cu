@@ -49,7 +49,6 @@ namespace {
 
 constexpr int AT_SOFTMAX = 8;  // softmax warps of a tile
 constexpr int AT_THREADS = 64 + 2 * 32 * AT_SOFTMAX;
-constexpr int AT_BANDS = 8;  // per CTA: two tiles of four
 constexpr int AT_BOX = 128 * 128;  // one 128-row x 128-byte swizzle box
 constexpr int AT_SMS = 152;
 

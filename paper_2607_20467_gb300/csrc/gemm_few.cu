@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   int* pos_s = reinterpret_cast<int*>(smem + FW_RING + 256);
   int* seq_s = pos_s + FEW_MAX_ROWS;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int S = (int)cluster_size(), rank = (int)cluster_rank();
   const int u = (int)blockIdx.x / S;  // the cluster's tile
   const int kb0 = rank * a.nkb / S, nkb = (rank + 1) * a.nkb / S - kb0;
@@ -291,28 +291,38 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && nt > 0) {
-      // ------------------------------------------------ MMA issuer
+    if (nt > 0) {
+      // ------------------------------------------------ MMA issuer (the whole warp, one lane issues)
       const uint32_t idesc = make_idesc(FW_TILE, nt);
+      const bool leader = elect_one();
       bool ok = true;
+      int stage = 0;
+      uint32_t phase = 0;
       for (int kb = 0; kb < nkb; ++kb) {
-        const int stage = kb % stages;
-        if (!mbar_wait(full0 + 8 * stage, (uint32_t)(kb / stages) & 1u, abort_flag)) {
+        if (!__all_sync(0xffffffffu, mbar_wait_inline(full0 + 8 * stage, phase, abort_flag))) {
           ok = false;
           break;
         }
-        const uint32_t sw = base + (uint32_t)(stage * stage_bytes);
-        const uint64_t dw = sw128_desc(sw), dx = sw128_desc(sw + FW_W_BYTES);
+        if (leader) {
+          const uint32_t sw = base + (uint32_t)(stage * stage_bytes);
+          const uint64_t dw = sw128_desc(sw), dx = sw128_desc(sw + FW_W_BYTES);
 #pragma unroll
-        for (int k = 0; k < FW_BK / 16; ++k)
-          umma_bf16(tmem_base, dw + 2 * k, dx + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
-        umma_commit(empty0 + 8 * stage);
+          for (int k = 0; k < FW_BK / 16; ++k)
+            umma_bf16(tmem_base, dw + 2 * k, dx + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          umma_commit(empty0 + 8 * stage);
+        }
+        __syncwarp();
+        if (++stage == stages) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
       if (!ok) {
         *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
+        if (leader) report_error(err, DERR_WAIT_TIMEOUT);
       }
-      umma_commit(done);  // (in either case every MMA issued here completes before TMEM is released)
+      if (leader) umma_commit(done);  // (in either case every MMA issued here completes before TMEM is released)
+      __syncwarp();
       volatile int no_abort = 0;
       mbar_wait(done, 0, &no_abort);
     }

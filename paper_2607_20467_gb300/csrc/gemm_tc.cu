@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int num_m = (M + BM - 1) / BM;
   const int num_n = (N + BN - 1) / BN;
   const int num_tiles = num_m * num_n;
@@ -293,50 +293,57 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------ MMA issuer
-      constexpr uint32_t idesc = make_idesc(BM, BN);
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      int j = 0;
-      for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++j) {
-        const int ab = j & 1;
-        const uint32_t aph = (uint32_t)(j >> 1) & 1u;
-        if (!mbar_wait(tempty0 + 8 * ab, aph ^ 1u, abort_flag)) {
+    // ------------------------------------------------ MMA issuer (the whole warp, one lane issues)
+    constexpr uint32_t idesc = make_idesc(BM, BN);
+    const bool leader = elect_one();
+    auto wait = [&](uint32_t bar, uint32_t parity) {
+      return (bool)__all_sync(0xffffffffu, mbar_wait_inline(bar, parity, abort_flag));
+    };
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    int j = 0;
+    for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x, ++j) {
+      const int ab = j & 1;
+      const uint32_t aph = (uint32_t)(j >> 1) & 1u;
+      if (!wait(tempty0 + 8 * ab, aph ^ 1u)) {
+        ok = false;
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(ab * BN);
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (!wait(full0 + 8 * stage, phase)) {
           ok = false;
           break;
         }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(ab * BN);
-        for (int kb = 0; kb < num_kb; ++kb) {
-          if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) {
-            ok = false;
-            break;
-          }
+        if (leader) {
           const uint64_t da = sw128_desc(sA + stage * A_STAGE_BYTES);
           const uint64_t db = sw128_desc(sB + stage * C::B_STAGE_BYTES);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k)  // advance 16 elements = 32 bytes = 2 desc units
             umma_bf16(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
           umma_commit(empty0 + 8 * stage);
-          if (++stage == C::STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
         }
-        if (!ok) break;
-        umma_commit(tfull0 + 8 * ab);
+        __syncwarp();
+        if (++stage == C::STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
-      }
-      // all MMAs issued by this thread complete before TMEM is released
-      umma_commit(drain);
-      volatile int no_abort = 0;
-      mbar_wait(drain, 0, &no_abort);
+      if (!ok) break;
+      if (leader) umma_commit(tfull0 + 8 * ab);
+      __syncwarp();
     }
+    if (!ok) {
+      *abort_flag = 1;
+      if (leader) report_error(err, DERR_WAIT_TIMEOUT);
+    }
+    // all MMAs issued by this warp complete before TMEM is released
+    if (leader) umma_commit(drain);
+    __syncwarp();
+    volatile int no_abort = 0;
+    mbar_wait(drain, 0, &no_abort);
   } else {
     // ------------------------------------------------ epilogue warps 2..5
     const int q = warp & 3;  // TMEM lane quarter this warp may access
@@ -1110,7 +1117,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const uint32_t crank = cluster_ctarank();
   const uint32_t rank = crank & 1u;             // 0: leader of the pair (issues the MMAs), 1: peer
   const uint32_t lead = crank & ~1u;            // cluster rank of this pair's leader
@@ -1242,10 +1249,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ------------------------------------------------ MMA issuer (leader CTA only)
+    if (rank == 0) {
+      // ------------------------------------------------ MMA issuer (leader CTA only; the whole
+      // warp, one lane issues: see elect_one)
       constexpr uint32_t idesc_full = make_idesc(256, 256);
       constexpr uint32_t idesc_half = make_idesc(256, 128);
+      const bool leader = elect_one();
+      auto wait = [&](uint32_t bar, uint32_t parity) {
+        return (bool)__all_sync(0xffffffffu, mbar_wait_inline(bar, parity, abort_flag));
+      };
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -1255,41 +1267,46 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const uint32_t idesc = it.width == 256 ? idesc_full : idesc_half;
         const int ab = idx & 1;
         const uint32_t aph = (uint32_t)(idx >> 1) & 1u;
-        if (!mbar_wait(tempty0 + 8 * ab, aph ^ 1u, abort_flag)) {
+        if (!wait(tempty0 + 8 * ab, aph ^ 1u)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(ab * 256);
         for (int kb = kb0; kb < kb1; kb += KA2) {
-          if (!mbar_wait(full0 + 8 * stage, phase, abort_flag)) {
+          if (!wait(full0 + 8 * stage, phase)) {
             ok = false;
             break;
           }
           // (no tcgen05 fence here: the stage was written by TMA, whose completion the
           // mbarrier itself publishes to the tensor core's async proxy)
+          if (leader) {
 #pragma unroll
-          for (int a = 0; a < KA2; ++a) {
-            const uint64_t da = sw128_desc(sA + stage * A2_STAGE_BYTES + a * A_STAGE_BYTES);
-            const uint64_t db = sw128_desc(sB + stage * B2_STAGE_BYTES + a * B2_BLOCK_BYTES);
+            for (int a = 0; a < KA2; ++a) {
+              const uint64_t da = sw128_desc(sA + stage * A2_STAGE_BYTES + a * A_STAGE_BYTES);
+              const uint64_t db = sw128_desc(sB + stage * B2_STAGE_BYTES + a * B2_BLOCK_BYTES);
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb > kb0 || a > 0 || k > 0) ? 1u : 0u);
+              for (int k = 0; k < BK / 16; ++k)
+                umma_bf16_pair(d_tmem, da + 2 * k, db + 2 * k, idesc, (kb > kb0 || a > 0 || k > 0) ? 1u : 0u);
+            }
+            umma_commit_pair(empty0 + 8 * stage, pair_mask);
           }
-          umma_commit_pair(empty0 + 8 * stage, pair_mask);
+          __syncwarp();
           if (++stage == STAGES2) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        umma_commit_pair(tfull0 + 8 * ab, pair_mask);
+        if (leader) umma_commit_pair(tfull0 + 8 * ab, pair_mask);
+        __syncwarp();
       }
       if (!ok) {
         *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
+        if (leader) report_error(err, DERR_WAIT_TIMEOUT);
       }
-      umma_commit_pair(drain, (uint16_t)(1u << lead));
+      if (leader) umma_commit_pair(drain, (uint16_t)(1u << lead));
+      __syncwarp();
       volatile int no_abort = 0;
       mbar_wait(drain, 0, &no_abort);
     }
