@@ -118,7 +118,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CUtensorMap tk,
                    const __grid_constant__ CUtensorMap tv, const __grid_constant__ CUtensorMap to,
                    __nv_bfloat16* __restrict__ out, int B, int T, int H, int G, int kcol0,
-                   const int* __restrict__ seq_off, const int* __restrict__ seq_len, int mode, int bands, int* err) {
+                   const int* __restrict__ seq_off, const int* __restrict__ seq_len, int q_rows, int mode, int bands,
+                   int* err) {
   using C = AttnCfg<HD>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -179,8 +180,9 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   pdl_wait();  // the previous kernels of the step (the row plan among them) have completed
   pdl_launch_dependents();
   // the query rows of sequence b are rows [off, off + len) of q and of the output
-  const int q_off = seq_off ? seq_off[b] : b * T;
-  const int q_len = seq_len ? seq_len[b] : T;
+  // (without tables its last q_rows positions)
+  const int q_off = seq_off ? seq_off[b] : b * T + T - q_rows;
+  const int q_len = seq_len ? seq_len[b] : q_rows;
   bool split = mode == ATTN_SPLIT;
   if (mode == ATTN_BY_ROWS) {
     // the cheapest of whole or split units of eight or four bands that the grid has CTAs for
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
           if (seq_off)
             tma_store_2d(&to, bx, col0 + c, q_off + row0);
           else
-            tma_store_3d(&to, bx, col0 + c, row0, b);
+            tma_store_3d(&to, bx, col0 + c, T - q_rows + row0, b);
         }
       }
       if (lane == 0) {
@@ -627,7 +629,7 @@ cudaError_t launch_attn(const AttnPlan& p, const AttnRows& rows, int* err, cudaS
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, p.tq, p.tk, p.tv, p.to, p.out, p.batch, p.T, p.H, p.G, p.kcol0, p.seq_off,
-                            p.seq_len, a.mode, a.bands, err);
+                            p.seq_len, rows.most, a.mode, a.bands, err);
 }
 
 }  // namespace

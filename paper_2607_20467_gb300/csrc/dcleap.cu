@@ -104,11 +104,24 @@ struct dcl_ctx {
   bool profiling = false;
   ProfGraph prof[STEP_BRANCHES];  // profiling: one graph per branch, the host takes the step's
   int prof_last = -1;             // the branch of the last profiled step
-  int32_t* h_done = nullptr;  // pinned [2]
+  // pinned: h_done [2], the error word's copy, and a buffer for the copies of the state and of
+  // the results (a copy from or to pageable memory waits for the stream each time)
+  int32_t* h_done = nullptr;
+  int32_t* h_err = nullptr;
+  int32_t* h_buf = nullptr;
+  // scratch of the single-kernel entry points, kept from call to call up to OP_SCRATCH_KEEP
+  void* op_buf = nullptr;
+  size_t op_cap = 0;
   cudaEvent_t ev_done[2] = {nullptr, nullptr};
 };
 
 namespace {
+
+// A single-kernel call's scratch of up to this size stays with the context (cudaMalloc and
+// cudaFree took 175 of the 288 us of an attention call whose kernels take 60); larger is
+// allocated and released by the call.
+constexpr size_t OP_SCRATCH_KEEP = 256u << 20;
+constexpr int PINNED_HEAD = 16;  // ints before h_buf
 
 dcl_status fail(dcl_ctx* c, dcl_status s, const char* fmt, ...) {
   char buf[512];
@@ -173,11 +186,11 @@ void dev_free_one(dcl_ctx* c, void* ptr) {
   }
 }
 
-// Read and clear the device error word; map it to a status.
+// Wait for the stream; read and clear the device error word; map it to a status.
 dcl_status check_device(dcl_ctx* c) {
-  int e = 0;
+  CUDA_TRY(c, cudaMemcpyAsync(c->h_err, c->derr, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  CUDA_TRY(c, cudaMemcpy(&e, c->derr, sizeof(int), cudaMemcpyDeviceToHost));
+  const int e = *c->h_err;
   if (e != DERR_NONE) {
     const int zero = 0;
     cudaMemcpy(c->derr, &zero, sizeof(int), cudaMemcpyHostToDevice);
@@ -190,6 +203,39 @@ dcl_status check_device(dcl_ctx* c) {
   }
   return DCL_OK;
 }
+
+// Scratch of one call of a single-kernel entry point: the context's (the calls on it run one
+// after another on its stream), or if larger than it keeps, the call's own.
+struct OpScratch {
+  dcl_ctx* c;
+  void* ptr = nullptr;
+  bool own = false;
+  explicit OpScratch(dcl_ctx* ctx) : c(ctx) {}
+  OpScratch(const OpScratch&) = delete;
+  bool get(size_t bytes) {
+    if (bytes == 0) return true;
+    if (bytes <= c->op_cap) {
+      ptr = c->op_buf;
+    } else if (bytes > OP_SCRATCH_KEEP) {
+      ptr = dev_alloc(c, bytes);
+      own = true;
+    } else {
+      if (c->op_buf) {
+        cudaStreamSynchronize(c->stream);  // no launch may still use the old buffer
+        dev_free_one(c, c->op_buf);
+      }
+      c->op_buf = dev_alloc(c, bytes);
+      c->op_cap = c->op_buf ? bytes : 0;
+      ptr = c->op_buf;
+    }
+    return ptr != nullptr;
+  }
+  ~OpScratch() {
+    if (!own || !ptr) return;
+    cudaStreamSynchronize(c->stream);
+    dev_free_one(c, ptr);
+  }
+};
 
 // ------------------------------------------------------------------ the step
 struct Enq {
@@ -328,9 +374,10 @@ dcl_status current_branch(dcl_ctx* c, int* out) {
     *out = step_branch(c->B * c->T);
     return DCL_OK;
   }
-  std::vector<int32_t> ph(c->B), pe(c->B);
-  CUDA_TRY(c, cudaMemcpyAsync(ph.data(), c->p, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(pe.data(), c->rp.pe_cache, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
+  int32_t* const ph = c->h_buf;
+  int32_t* const pe = ph + c->B;
+  CUDA_TRY(c, cudaMemcpyAsync(ph, c->p, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(pe, c->rp.pe_cache, 4 * (size_t)c->B, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   const int Bk = c->dcfg.block_len;
   long rows = 0;
@@ -646,37 +693,18 @@ dcl_status build_plans(dcl_ctx* c) {
   return DCL_OK;
 }
 
-// Scratch for a one-off GEMM launch (the single-kernel entry points): allocated here,
-// released by release_scratch after the launch has completed.
-void release_scratch(dcl_ctx* c, GemmPlan* p);
+// Scratch of a one-off GEMM launch (the single-kernel entry points): zeroed counters, then the
+// workspace, at mem (256-byte aligned).
+size_t gemm_scratch_bytes(const GemmPlan& p) { return align_up(sizeof(int) * p.flags_needed, 256) + sizeof(float) * p.ws_needed; }
 
-dcl_status attach_scratch(dcl_ctx* c, GemmPlan* p) {
-  if (p->flags_needed) {
-    p->flags = static_cast<int*>(dev_alloc(c, sizeof(int) * p->flags_needed));
-    if (!p->flags) return fail(c, DCL_ERR_OOM, "split-K counter allocation failed");
-    CUDA_TRY(c, cudaMemsetAsync(p->flags, 0, sizeof(int) * p->flags_needed, c->stream));
-  }
-  if (p->ws_needed) {
-    p->ws = static_cast<float*>(dev_alloc(c, sizeof(float) * p->ws_needed));
-    if (!p->ws) {
-      dev_free_one(c, p->flags);
-      p->flags = nullptr;
-      return fail(c, DCL_ERR_OOM, "split-K workspace allocation failed");
-    }
-  }
-  if (gemm_bind_scratch(p, p->flags, p->ws) != cudaSuccess) {
-    release_scratch(c, p);
-    return fail(c, DCL_ERR_CUDA, "GEMM scratch binding failed");
-  }
+dcl_status attach_scratch(dcl_ctx* c, GemmPlan* p, void* mem) {
+  int* flags = p->flags_needed ? static_cast<int*>(mem) : nullptr;
+  float* ws = nullptr;
+  if (p->ws_needed)
+    ws = reinterpret_cast<float*>(static_cast<uint8_t*>(mem) + align_up(sizeof(int) * p->flags_needed, 256));
+  if (flags) CUDA_TRY(c, cudaMemsetAsync(flags, 0, sizeof(int) * p->flags_needed, c->stream));
+  if (gemm_bind_scratch(p, flags, ws) != cudaSuccess) return fail(c, DCL_ERR_CUDA, "GEMM scratch binding failed");
   return DCL_OK;
-}
-
-void release_scratch(dcl_ctx* c, GemmPlan* p) {
-  cudaStreamSynchronize(c->stream);
-  dev_free_one(c, p->flags);
-  dev_free_one(c, p->ws);
-  p->flags = nullptr;
-  p->ws = nullptr;
 }
 
 // weight destination for (kind, layer): pointer, rows, and the gate/up interleave offset
@@ -726,7 +754,8 @@ dcl_status validate_ids(dcl_ctx* c, const int32_t* ids, size_t n) {
 dcl_status reset_done_count(dcl_ctx* c, const int32_t* p_host) {
   int32_t n = 0;
   for (int b = 0; b < c->B; ++b) n += p_host[b] >= c->T;
-  CUDA_TRY(c, cudaMemcpyAsync(c->done_count, &n, sizeof n, cudaMemcpyHostToDevice, c->stream));
+  c->h_done[0] = n;
+  CUDA_TRY(c, cudaMemcpyAsync(c->done_count, &c->h_done[0], sizeof n, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return DCL_OK;
 }
@@ -889,7 +918,9 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
       return fail(nullptr, DCL_ERR_CUDA, "RoPE table upload failed");
     }
   }
-  if (cudaMallocHost(&c->h_done, 2 * sizeof(int32_t)) != cudaSuccess ||
+  // h_buf: ids, positions and committed flags of a state; the results of a generation
+  const size_t hb = cfg ? (size_t)max_batch * max_seq * 5 + (size_t)max_batch * 16 : 0;
+  if (cudaMallocHost(&c->h_done, PINNED_HEAD * sizeof(int32_t) + hb) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_done[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->ev_done[1], cudaEventDisableTiming) != cudaSuccess) {
     dev_free_all(c);
@@ -897,6 +928,8 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
     delete c;
     return fail(nullptr, DCL_ERR_CUDA, "pinned host buffer / event creation failed");
   }
+  c->h_err = c->h_done + 2;
+  c->h_buf = c->h_done + PINNED_HEAD;
   *out = c;
   return DCL_OK;
 }
@@ -1058,20 +1091,21 @@ dcl_status dcl_generate(dcl_ctx* c, int32_t max_steps, int32_t* out, dcl_stats* 
       if (c->h_done[slot ^ 1] >= c->B) done = true;
     }
   }
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  if (launched > 0 && c->h_done[(launched - 1) & 1] >= c->B) done = true;
+  // the results in one wait: p, steps and the entropy bound of every row, then its tokens
+  int32_t* const ph = c->h_buf;
+  int32_t* const sh = ph + c->B;
+  float* const jh = reinterpret_cast<float*>(sh + c->B);
+  int32_t* const xh = sh + 2 * c->B;
+  CUDA_TRY(c, cudaMemcpyAsync(ph, c->p, 4 * c->B, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(sh, c->steps, 4 * c->B, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(jh, c->jpde, 4 * c->B, cudaMemcpyDeviceToHost, c->stream));
+  if (out)
+    CUDA_TRY(c, cudaMemcpy2DAsync(xh, 4 * (size_t)c->M, c->x + c->N, 4 * (size_t)c->T, 4 * (size_t)c->M, c->B,
+                                  cudaMemcpyDeviceToHost, c->stream));
   dcl_status s = check_device(c);
+  if (launched > 0 && c->h_done[(launched - 1) & 1] >= c->B) done = true;
   if (s != DCL_OK) return s;
-  std::vector<int32_t> ph(c->B), sh(c->B);
-  std::vector<float> jh(c->B);
-  CUDA_TRY(c, cudaMemcpy(ph.data(), c->p, 4 * c->B, cudaMemcpyDeviceToHost));
-  CUDA_TRY(c, cudaMemcpy(sh.data(), c->steps, 4 * c->B, cudaMemcpyDeviceToHost));
-  CUDA_TRY(c, cudaMemcpy(jh.data(), c->jpde, 4 * c->B, cudaMemcpyDeviceToHost));
-  if (out) {
-    for (int b = 0; b < c->B; ++b)
-      CUDA_TRY(c, cudaMemcpy(out + (size_t)b * c->M, c->x + (size_t)b * c->T + c->N, 4 * c->M,
-                             cudaMemcpyDeviceToHost));
-  }
+  if (out) memcpy(out, xh, 4 * (size_t)c->B * c->M);
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
   if (st) {
     int64_t tok = 0, stp = 0;
@@ -1125,13 +1159,18 @@ dcl_status dcl_set_state(dcl_ctx* c, const int32_t* x, const int32_t* p) {
     if (p[b] < c->N || p[b] > c->T) return fail(c, DCL_ERR_INVALID_ARG, "p[%d] = %d outside [N, N+M]", b, p[b]);
   // committed flags (read by the threshold rule only): every position before p, and every
   // later position that holds a token other than MASK
-  std::vector<uint8_t> ch((size_t)c->B * c->T);
+  const size_t n = (size_t)c->B * c->T;
+  int32_t* const xh = c->h_buf;  // (free: every call that uses it waits before it returns)
+  int32_t* const ph = xh + n;
+  uint8_t* const ch = reinterpret_cast<uint8_t*>(ph + c->B);
+  memcpy(xh, x, 4 * n);
+  memcpy(ph, p, 4 * (size_t)c->B);
   for (int b = 0; b < c->B; ++b)
     for (int i = 0; i < c->T; ++i)
       ch[(size_t)b * c->T + i] = (i < p[b] || x[(size_t)b * c->T + i] != c->cfg.mask_id) ? 1 : 0;
-  CUDA_TRY(c, cudaMemcpyAsync(c->cmt, ch.data(), ch.size(), cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->x, x, 4 * (size_t)c->B * c->T, cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->p, p, 4 * (size_t)c->B, cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->cmt, ch, n, cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->x, xh, 4 * n, cudaMemcpyHostToDevice, c->stream));
+  CUDA_TRY(c, cudaMemcpyAsync(c->p, ph, 4 * (size_t)c->B, cudaMemcpyHostToDevice, c->stream));
   CUDA_TRY(c, cudaMemsetAsync(c->rp.pe_cache, 0xff, 4 * (size_t)c->B, c->stream));  // the next step refreshes
   CUDA_TRY(c, cudaMemsetAsync(c->jpde, 0, 4 * (size_t)c->B, c->stream));
   return reset_done_count(c, p);
@@ -1143,6 +1182,7 @@ namespace {
 dcl_status forward_debug_impl(dcl_ctx* c, int layer, const float* h_in, bool commit, void* logits_dev,
                               int32_t* top1_dev, float* p1_dev, float* p2_dev, float* conf_dev, float* entropy_dev) {
   const size_t R = (size_t)c->B * c->T;
+  OpScratch mem(c);
   if (!c->snap || c->snap_rows < R) {
     c->snap = (float*)dev_alloc(c, sizeof(float) * (c->cfg.n_layers + 1) * R * c->cfg.d_model);
     if (!c->snap) return fail(c, DCL_ERR_OOM, "snapshot buffer allocation failed");
@@ -1172,10 +1212,10 @@ dcl_status forward_debug_impl(dcl_ctx* c, int layer, const float* h_in, bool com
     const char* why = nullptr;
     if (gemm_plan(&pl, c->xg, (int)G, c->cfg.d_model, c->lm_head, c->cfg.vocab, EPI_BF16, ep, c->num_sms, 0, &why))
       return fail(c, DCL_ERR_UNSUPPORTED, "logits plan: %s", why ? why : "?");
-    dcl_status s = attach_scratch(c, &pl);
+    if (!mem.get(gemm_scratch_bytes(pl))) return fail(c, DCL_ERR_OOM, "logits scratch allocation failed");
+    dcl_status s = attach_scratch(c, &pl, mem.ptr);
     if (s != DCL_OK) return s;
     const cudaError_t e = gemm_launch(pl, c->derr, c->stream);
-    release_scratch(c, &pl);
     if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "logits GEMM: %s", cudaGetErrorString(e));
   }
   return check_device(c);
@@ -1285,10 +1325,11 @@ dcl_status dcl_op_linear(dcl_ctx* c, const void* a_dev, const void* w_dev, void*
       return check_device(c);
     }
   }
-  dcl_status s = attach_scratch(c, &pl);
+  OpScratch mem(c);
+  if (!mem.get(gemm_scratch_bytes(pl))) return fail(c, DCL_ERR_OOM, "GEMM scratch allocation failed");
+  dcl_status s = attach_scratch(c, &pl, mem.ptr);
   if (s != DCL_OK) return s;
   const cudaError_t e = gemm_launch(pl, c->derr, c->stream);
-  release_scratch(c, &pl);
   if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "GEMM launch: %s", cudaGetErrorString(e));
   return check_device(c);
 }
@@ -1299,45 +1340,22 @@ dcl_status dcl_op_attention(dcl_ctx* c, const void* qkv_dev, void* out_dev, int3
   if (!qkv_dev || !out_dev || batch <= 0 || T <= 0 || H <= 0 || G <= 0 || H % G || (hd != 64 && hd != 128) ||
       q_rows < 0 || q_rows > T || q_rows % 32)
     return fail(c, DCL_ERR_INVALID_ARG, "bad attention args");
-  __half* vt = static_cast<__half*>(dev_alloc(c, 2 * (size_t)batch * G * hd * attn_vt_pitch(T)));
-  int* tab = q_rows > 0 ? static_cast<int*>(dev_alloc(c, sizeof(int) * 2 * (size_t)batch)) : nullptr;
-  auto release = [&]() {
-    cudaStreamSynchronize(c->stream);
-    dev_free_one(c, vt);
-    dev_free_one(c, tab);
-  };
-  if (!vt || (q_rows > 0 && !tab)) {
-    release();
+  OpScratch mem(c);
+  if (!mem.get(2 * (size_t)batch * G * hd * attn_vt_pitch(T)))
     return fail(c, DCL_ERR_OOM, "attention scratch allocation failed");
-  }
-  if (tab) {  // sequence b's queries: positions [T - q_rows, T), rows b*T + T - q_rows onwards
-    std::vector<int> th(2 * (size_t)batch);
-    for (int b = 0; b < batch; ++b) {
-      th[b] = b * T + T - q_rows;
-      th[batch + b] = q_rows;
-    }
-    CUDA_TRY(c, cudaMemcpyAsync(tab, th.data(), sizeof(int) * th.size(), cudaMemcpyHostToDevice, c->stream));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  }
   AttnPlan pl;
-  if (attention_plan(&pl, static_cast<const __nv_bfloat16*>(qkv_dev), nullptr, vt, static_cast<__nv_bfloat16*>(out_dev),
-                     batch, T, H, G, hd, batch * T, tab, tab ? tab + batch : nullptr) != cudaSuccess) {
-    release();
+  if (attention_plan(&pl, static_cast<const __nv_bfloat16*>(qkv_dev), nullptr, static_cast<__half*>(mem.ptr),
+                     static_cast<__nv_bfloat16*>(out_dev), batch, T, H, G, hd, batch * T, nullptr, nullptr) !=
+      cudaSuccess)
     return fail(c, DCL_ERR_INVALID_ARG, "attention: operands must be 16-byte aligned");
-  }
-  AttnRows ar;
+  AttnRows ar;  // sequence b's queries: positions [T - q_rows, T)
   ar.most = q_rows ? q_rows : T;
   ar.total = batch * ar.most;
   ar.seqs = batch;
   ar.exact = true;
   const cudaError_t e = attention_launch(pl, ar, c->derr, c->stream);
-  if (e != cudaSuccess) {
-    release();
-    return fail(c, DCL_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
-  }
-  const dcl_status s = check_device(c);
-  release();
-  return s;
+  if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "attention launch: %s", cudaGetErrorString(e));
+  return check_device(c);
 }
 
 dcl_status dcl_op_lmhead_top2(dcl_ctx* c, const void* x_dev, const void* w_dev, int32_t R, int32_t V, int32_t d,
@@ -1348,38 +1366,29 @@ dcl_status dcl_op_lmhead_top2(dcl_ctx* c, const void* x_dev, const void* w_dev, 
   if (tile != 0 && tile != 256 && (tile & 0xff) != kTilePair) return fail(c, DCL_ERR_INVALID_ARG, "bad tile");
   const int nblk = gemm_lmhead_blocks(V);
   // {max, sum, id, second} partials, then (with entropy_dev) the entropy partials
-  float4* part = static_cast<float4*>(dev_alloc(c, (sizeof(float4) + (entropy_dev ? 4 : 0)) * (size_t)R * nblk));
-  if (!part) return fail(c, DCL_ERR_OOM, "partials allocation failed");
-  float* upart = entropy_dev ? reinterpret_cast<float*>(part + (size_t)R * nblk) : nullptr;
+  const size_t part_bytes = align_up((sizeof(float4) + (entropy_dev ? 4 : 0)) * (size_t)R * nblk, 256);
   GemmPlan pl;
   EpiParams ep;
-  ep.out = part;
-  ep.ent_part = upart;
   const char* why = nullptr;
-  if (gemm_plan(&pl, x_dev, R, d, w_dev, V, EPI_LMHEAD, ep, c->num_sms, tile, &why)) {
-    dev_free_one(c, part);
+  if (gemm_plan(&pl, x_dev, R, d, w_dev, V, EPI_LMHEAD, ep, c->num_sms, tile, &why))
     return fail(c, DCL_ERR_INVALID_ARG, "%s", why ? why : "bad LM-head shape");
-  }
-  dcl_status s = attach_scratch(c, &pl);
-  if (s != DCL_OK) {
-    dev_free_one(c, part);
-    return s;
-  }
+  OpScratch mem(c);
+  if (!mem.get(part_bytes + gemm_scratch_bytes(pl))) return fail(c, DCL_ERR_OOM, "partials allocation failed");
+  float4* part = static_cast<float4*>(mem.ptr);
+  float* upart = entropy_dev ? reinterpret_cast<float*>(part + (size_t)R * nblk) : nullptr;
+  pl.ep.out = part;
+  pl.ep.ent_part = upart;
+  dcl_status s = attach_scratch(c, &pl, static_cast<uint8_t*>(mem.ptr) + part_bytes);
+  if (s != DCL_OK) return s;
   const cudaError_t e = gemm_launch(pl, c->derr, c->stream);
-  release_scratch(c, &pl);
-  if (e != cudaSuccess) {
-    dev_free_one(c, part);
-    return fail(c, DCL_ERR_CUDA, "LM-head GEMM: %s", cudaGetErrorString(e));
-  }
+  if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "LM-head GEMM: %s", cudaGetErrorString(e));
   ConfOut co;
   co.top1 = top1_dev;
   co.p1 = p1_dev;
   co.p2 = p2_dev;
   co.ent = entropy_dev;
   CUDA_TRY(c, lmhead_combine_launch(part, upart, R, nblk, co, nullptr, nullptr, c->stream));
-  s = check_device(c);
-  dev_free_one(c, part);
-  return s;
+  return check_device(c);
 }
 
 dcl_status dcl_op_generate(dcl_ctx* c, void* dst_dev, uint64_t seed, int32_t tid, int64_t start, int64_t count,
