@@ -170,9 +170,10 @@ bool encode_tmap(CUtensorMap* tm, CUtensorMapDataType dt, int rank, void* ptr, c
                  const uint64_t* strides, const uint32_t* box, CUtensorMapSwizzle swizzle);
 
 // ---------------------------------------------------------------- few-row GEMM (gemm_few.cu)
-// out = X[M][K] @ W[N][K]^T for at most FEW_MAX_ROWS rows, weight rows on the MMA's M side
-// and the rows of X on its N side; epilogues EPI_BF16, EPI_RESID_F32, EPI_QKV_ROPE, EPI_SWIGLU.
-constexpr int FEW_MAX_ROWS = 128;
+// out = X[M][K] @ W[N][K]^T for few rows of X, weight rows on the MMA's M side and up to
+// FEW_TILE_ROWS rows of X on its N side; epilogues EPI_BF16, EPI_RESID_F32, EPI_QKV_ROPE,
+// EPI_SWIGLU.
+constexpr int FEW_TILE_ROWS = 128;
 struct FewEpi {
   void* out = nullptr;             // as EpiParams::out (with QKV: q, and k / v without the stores below)
   int ldo = 0;
@@ -189,12 +190,16 @@ struct FewEpi {
 struct FewPlan {
   CUtensorMap tw, tx;
   int M = 0, N = 0, K = 0, epi = EPI_BF16;
-  int nt_max = 0;  // the rows a launch may hold: 32 or FEW_MAX_ROWS (fewer give a deeper ring)
-  int units = 0, split = 1;  // tiles of 128 weight rows, CTAs (a cluster) that share a tile's K
+  int nt_max = 0;  // the rows of a token tile: 32 or FEW_TILE_ROWS (fewer give a deeper ring)
+  int units = 0, tiles = 1, split = 1;  // tiles of 128 weight rows, of tokens; CTAs (a cluster) that share one's K
   FewEpi ep;
 };
+// rows: the most rows a launch may hold (<= M).
 cudaError_t few_plan(FewPlan* plan, const void* X, int M, int K, const void* W, int N, int epi, const FewEpi& ep,
-                     int num_sms, int nt_max);
+                     int num_sms, int rows);
+// Up to how many rows of X the few-row GEMM is taken for N weight rows: while its tiles fit the
+// GPU at once (two CTAs per SM), and for one token tile in any case.
+int few_rows(int N, int num_sms);
 cudaError_t few_launch(const FewPlan& plan, int* err, cudaStream_t stream);
 
 // ---------------------------------------------------------------- attention (attention_tc.cu)
@@ -256,11 +261,12 @@ struct RowPlan {
 // select: the conditional node that takes the step's branch (StepBranch of the row count), or 0.
 cudaError_t row_plan_launch(const RowPlan& rp, const int32_t* p, int batch, int N, int T, int block_len,
                             int cached, int update, int32_t* x, int window, int mask_id,
-                            cudaGraphConditionalHandle select, cudaStream_t stream);
-// The GEMM kernels of a step, by the rows it computes.
+                            cudaGraphConditionalHandle select, int few_max, cudaStream_t stream);
+// The GEMM kernels of a step, by the rows it computes (few_max: the most that the shape's
+// few-row GEMMs take).
 enum StepBranch : int { STEP_PAIR = 0, STEP_FEW32 = 1, STEP_FEW = 2, STEP_BRANCHES = 3 };
-__host__ __device__ inline int step_branch(int rows) {
-  return rows <= 32 ? STEP_FEW32 : rows <= FEW_MAX_ROWS ? STEP_FEW : STEP_PAIR;
+__host__ __device__ inline int step_branch(int rows, int few_max) {
+  return rows <= 32 ? STEP_FEW32 : rows <= few_max ? STEP_FEW : STEP_PAIR;
 }
 cudaError_t embed_remask_launch(int32_t* x, const int32_t* p, int batch, int T, int window,
                                 int mask_id, int vocab, const __nv_bfloat16* embed, int d,

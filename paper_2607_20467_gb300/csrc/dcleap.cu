@@ -98,8 +98,9 @@ struct dcl_ctx {
   std::vector<AttnPlan> attn_plans;  // one per layer
   bool kv_fused = false;  // the QKV GEMMs write k and v^T (no transpose launch)
   // few-row GEMMs of the layers (qkv, o, gate/up, down; 4 per layer): [0] for up to 32 rows,
-  // [1] for up to FEW_MAX_ROWS; empty where no step of this shape takes them
+  // [1] for up to few_max; empty where no step of this shape takes them
   std::vector<FewPlan> few[2];
+  int few_max = 0;
   cudaGraphExec_t gexec = nullptr;
   bool profiling = false;
   ProfGraph prof[STEP_BRANCHES];  // profiling: one graph per branch, the host takes the step's
@@ -271,7 +272,7 @@ struct Enq {
 void enqueue_rows(dcl_ctx* c, Enq& q, bool update, cudaGraphConditionalHandle select) {
   q.begin(DCL_K_ROWPLAN);
   q.end(row_plan_launch(c->rp, c->p, c->B, c->N, c->T, c->dcfg.block_len, c->dcfg.kv_cache, update ? 1 : 0, c->x,
-                        c->dcfg.acceptance ? 0 : c->window, c->cfg.mask_id, select, c->stream),
+                        c->dcfg.acceptance ? 0 : c->window, c->cfg.mask_id, select, c->few_max, c->stream),
         "row_plan");
 }
 
@@ -284,7 +285,7 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
   const int R = c->B * c->T;
   const int d = m.d_model;
   const std::vector<FewPlan>* few = branch == STEP_PAIR ? nullptr : &c->few[branch == STEP_FEW32 ? 0 : 1];
-  const int rows = std::min(R, branch == STEP_FEW32 ? 32 : branch == STEP_FEW ? FEW_MAX_ROWS : R);  // at most
+  const int rows = std::min(R, branch == STEP_FEW32 ? 32 : branch == STEP_FEW ? c->few_max : R);  // at most
   AttnRows ar;  // the attention's query rows: every position, or as the row plan says
   ar.most = std::min(c->T, rows);
   ar.total = rows;
@@ -371,7 +372,7 @@ dcl_status current_branch(dcl_ctx* c, int* out) {
   *out = STEP_PAIR;
   if (c->few[0].empty()) return DCL_OK;
   if (!c->dcfg.kv_cache) {
-    *out = step_branch(c->B * c->T);
+    *out = step_branch(c->B * c->T, c->few_max);
     return DCL_OK;
   }
   int32_t* const ph = c->h_buf;
@@ -388,7 +389,7 @@ dcl_status current_branch(dcl_ctx* c, int* out) {
     const int start = fresh ? end : 0;
     rows += (c->dcfg.kv_cache == 2 && start != 0 ? std::min(end + Bk, c->T) : c->T) - start;
   }
-  *out = step_branch((int)rows);
+  *out = step_branch((int)rows, c->few_max);
   return DCL_OK;
 }
 
@@ -459,7 +460,7 @@ dcl_status build_exec(dcl_ctx* c, cudaGraphExec_t* exec, bool with_switch, int b
 dcl_status build_graph(dcl_ctx* c) {
   destroy_graphs(c);
   const bool by_rows = !c->few[0].empty() && c->dcfg.kv_cache;
-  const int fixed = c->few[0].empty() ? (int)STEP_PAIR : step_branch(c->B * c->T);
+  const int fixed = c->few[0].empty() ? (int)STEP_PAIR : step_branch(c->B * c->T, c->few_max);
   if (!c->profiling) return build_exec(c, &c->gexec, by_rows, fixed, nullptr);
   for (int br = 0; br < STEP_BRANCHES; ++br)
     if (by_rows || br == fixed) {
@@ -621,10 +622,11 @@ dcl_status build_plans(dcl_ctx* c) {
   c->few[0].clear();
   c->few[1].clear();
   const bool planned = t_qkv == kTilePair && t_o == kTilePair && t_gu == kTilePair && t_down == kTilePair;
-  if (planned && (cached || R <= FEW_MAX_ROWS)) {
+  c->few_max = few_rows(std::max(std::max(nqkv, d), 2 * m.ffn_dim), c->num_sms);
+  if (planned && (cached || R <= c->few_max)) {
     bool ok = true;
     for (int v = 0; v < 2 && ok; ++v) {
-      const int nt = v == 0 ? 32 : FEW_MAX_ROWS;
+      const int nt = std::min(R, v == 0 ? 32 : c->few_max);
       c->few[v].assign(4 * m.n_layers, FewPlan{});
       for (int l = 0; l < m.n_layers && ok; ++l) {
         const Layer& L = c->layers[l];
@@ -1313,13 +1315,13 @@ dcl_status dcl_op_linear(dcl_ctx* c, const void* a_dev, const void* w_dev, void*
   const char* why = nullptr;
   if (gemm_plan(&pl, a_dev, M, K, w_dev, N, mode == 0 ? EPI_BF16 : EPI_RESID_F32, ep, c->num_sms, tile, &why))
     return fail(c, DCL_ERR_INVALID_ARG, "%s", why ? why : "bad GEMM shape");
-  if (tile == 0 && M <= FEW_MAX_ROWS) {  // as the step's GEMMs of so few rows
+  if (tile == 0 && M <= FEW_TILE_ROWS) {  // as the step's GEMMs of so few rows
     FewPlan fp;
     FewEpi fe;
     fe.out = out_dev;
     fe.ldo = N;
     if (few_plan(&fp, a_dev, M, K, w_dev, N, mode == 0 ? EPI_BF16 : EPI_RESID_F32, fe, c->num_sms,
-                 M <= 32 ? 32 : FEW_MAX_ROWS) == cudaSuccess) {
+                 M) == cudaSuccess) {
       const cudaError_t e = few_launch(fp, c->derr, c->stream);
       if (e != cudaSuccess) return fail(c, DCL_ERR_CUDA, "GEMM launch: %s", cudaGetErrorString(e));
       return check_device(c);

@@ -1,4 +1,4 @@
-// GEMMs of a step with few rows (at most FEW_MAX_ROWS tokens: the current block or a short
+// GEMMs of a step with few rows (the current block or a short
 // suffix under the key / value caches, small full recomputes):
 //   out = X[rows][K] @ W[N][K]^T   with the step's epilogues fused.
 //
@@ -24,8 +24,14 @@
 // bytes in flight) stream faster: 192 CTAs of the gate/up GEMM read 201 MB in 29 us (6.9
 // TB/s), 96 CTAs of an unsplit QKV 100 MB in 22 us, 192 in 16 us.
 //
+// Where the weights are small (few_rows) more rows are taken too, as tiles of 128 tokens beside
+// each other: while all tiles fit the GPU at once a launch is latency, and these are shorter
+// than the pair kernel's (a fused MLP took 27 us at d 768, ffn 2048).
+//
 // Measured per step, 8 layers of the LLaDA-8B shape at T = 1536: 32 rows 1415 -> 1092 us, 96
-// rows 1430 -> 1208 us; the 2-layer test model (96 rows, latency) 119 -> 81 us.
+// rows 1430 -> 1208 us; the 2-layer test model (96 rows, latency) 119 -> 81 us; four layers of
+// d 768, ffn 2048: 192 rows 254 -> 214 us, 512 rows 260 -> 231, 1024 rows 278 -> 243 (at 1536
+// rows, past one round of tiles, the pair kernels take 299).
 #include <string.h>
 
 #include <algorithm>
@@ -42,16 +48,17 @@ constexpr int FW_TILE = 128;              // weight rows of a tile
 constexpr int FW_W_BYTES = FW_TILE * 128; // a K block of them
 constexpr int FW_XBOX_BYTES = 32 * 128;   // 32 tokens x one K block
 constexpr int FW_MAX_STAGES = 5;
-constexpr int FW_BARS = 256 + 2 * 4 * FEW_MAX_ROWS;  // barriers, then the tokens' positions and sequences
+constexpr int FW_BARS = 256 + 2 * 4 * FEW_TILE_ROWS;  // barriers, then the tokens' positions and sequences
 constexpr size_t FW_SMEM = 112 * 1024;
 constexpr int FW_RING = (int)FW_SMEM - 1024 - FW_BARS;
 constexpr int FW_PITCH = FW_TILE + 4;     // fp32 per token of a staged sum
-static_assert(FEW_MAX_ROWS * FW_PITCH * 4 <= FW_RING, "the staged sum lives in the operand ring");
+static_assert(FEW_TILE_ROWS * FW_PITCH * 4 <= FW_RING, "the staged sum lives in the operand ring");
 static_assert(8 * (2 * FW_MAX_STAGES + 1) + 16 <= 256, "barrier area");
 
 struct FewArgs {
   int nkb;     // K blocks
-  int nt_max;  // tokens the launch may hold (32 or FEW_MAX_ROWS)
+  int nt_max;  // tokens of a token tile at most (32 or FEW_TILE_ROWS)
+  int units, tiles;
   int N, M;
   FewEpi ep;
 };
@@ -97,7 +104,7 @@ __device__ __forceinline__ void store_bf16x4(__nv_bfloat16* o, float a, float b,
 // thread.  sum: the staged sums [token][FW_PITCH], at the same shared address in each of the
 // cluster's S CTAs.
 template <int EPI, int S>
-__device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u, int t0, int t1, int et,
+__device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u, int tok0, int t0, int t1, int et,
                                            const int* pos_s, const int* seq_s) {
   const FewEpi& ep = a.ep;
   const int n0 = u * FW_TILE;
@@ -115,7 +122,7 @@ __device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
         if (i >= m) continue;
-        const size_t o = (size_t)(t + 4 * i) * ep.ldo + n;
+        const size_t o = (size_t)(tok0 + t + 4 * i) * ep.ldo + n;
         if constexpr (EPI == EPI_BF16)
           store_bf16x4(static_cast<__nv_bfloat16*>(ep.out) + o, x[i].x, x[i].y, x[i].z, x[i].w);
         else
@@ -134,7 +141,7 @@ __device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u
 #pragma unroll
       for (int i = 0; i < NP; ++i)
         if (i < m)
-          store_bf16x4(static_cast<__nv_bfloat16*>(ep.out) + (size_t)(t + 8 * i) * ep.ldo + u * 64 + j,
+          store_bf16x4(static_cast<__nv_bfloat16*>(ep.out) + (size_t)(tok0 + t + 8 * i) * ep.ldo + u * 64 + j,
                        act(g[i].x, v[i].x), act(g[i].y, v[i].y), act(g[i].z, v[i].z), act(g[i].w, v[i].w));
     }
   } else if (n0 >= ep.rope_cols && ep.vdst) {
@@ -181,7 +188,7 @@ __device__ __forceinline__ void few_finish(const FewArgs& a, uint32_t sum, int u
         if (i >= m) continue;
         const int tt = t + 8 * i;
         __nv_bfloat16* o = to_k ? ep.kdst + ((size_t)seq_s[tt] * ep.T + pos_s[tt]) * ep.G * ep.head_dim + (n0 - ep.k_col0)
-                                : static_cast<__nv_bfloat16*>(ep.out) + (size_t)tt * ep.ldo + n0;
+                                : static_cast<__nv_bfloat16*>(ep.out) + (size_t)(tok0 + tt) * ep.ldo + n0;
         store_bf16x4(o + r0, x[i].x * c[i].x - y[i].x * c[i].y, x[i].y * c[i].z - y[i].y * c[i].w,
                      x[i].z * d[i].x - y[i].z * d[i].y, x[i].w * d[i].z - y[i].w * d[i].w);
         store_bf16x4(o + r1, y[i].x * c[i].x + x[i].x * c[i].y, y[i].y * c[i].z + x[i].y * c[i].w,
@@ -204,11 +211,12 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
   int* pos_s = reinterpret_cast<int*>(smem + FW_RING + 256);
-  int* seq_s = pos_s + FEW_MAX_ROWS;
+  int* seq_s = pos_s + FEW_TILE_ROWS;
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int S = (int)cluster_size(), rank = (int)cluster_rank();
-  const int u = (int)blockIdx.x / S;  // the cluster's tile
+  // the cluster's tile of weight rows and its tile of tokens (rows [tok0, tok0 + nt_max))
+  const int u = (int)blockIdx.x / S % a.units, tok0 = (int)blockIdx.x / S / a.units * a.nt_max;
   const int kb0 = rank * a.nkb / S, nkb = (rank + 1) * a.nkb / S - kb0;
   // a stage: the weight rows of one K block, then the tokens'.  The stage pitch is that of
   // the most tokens the launch may hold, known before the row count is.
@@ -244,7 +252,7 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
       mbar_expect_tx(full0 + 8 * pre, FW_W_BYTES);
       load_w(pre, pre);
     }
-  if (warp == 1) tmem_alloc(holder, FEW_MAX_ROWS);
+  if (warp == 1) tmem_alloc(holder, FEW_TILE_ROWS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -252,9 +260,10 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
 
   pdl_wait();
   pdl_launch_dependents();
-  const int rows = a.ep.m_dev ? min(a.M, *a.ep.m_dev) : a.M;
-  int nt = (rows + 31) & ~31;  // the MMA's N
-  if (nt > a.nt_max) {         // (the launch is not chosen for so many rows)
+  const int all = a.ep.m_dev ? min(a.M, *a.ep.m_dev) : a.M;
+  const int rows = max(min(all - tok0, a.nt_max), 0);
+  int nt = (rows + 31) & ~31;         // the MMA's N
+  if (all > a.tiles * a.nt_max) {     // (the launch is not chosen for so many rows)
     if (threadIdx.x == 0) report_error(err, DERR_BAD_SHAPE);
     nt = 0;
   }
@@ -275,7 +284,7 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
         if (!have_w) load_w(stage, kb);
         for (int b = 0; b < nt / 32; ++b)
           tma_load_2d(base + (uint32_t)(stage * stage_bytes + FW_W_BYTES + b * FW_XBOX_BYTES), &tx, (kb0 + kb) * FW_BK,
-                      b * 32, full0 + 8 * stage);
+                      tok0 + b * 32, full0 + 8 * stage);
         ++issued;
       }
       if (!ok) {
@@ -330,8 +339,8 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
     // ------------------------------------------------ epilogue warps 2..5: the sum to shared memory
     const int et = threadIdx.x - 64;
     if (EPI == EPI_QKV_ROPE && et < rows) {
-      pos_s[et] = a.ep.row_pos[et];
-      seq_s[et] = a.ep.row_seq[et];
+      pos_s[et] = a.ep.row_pos[tok0 + et];
+      seq_s[et] = a.ep.row_seq[tok0 + et];
     }
     const int q = warp & 3;  // TMEM lane quarter: rows 32 q .. 32 q + 31 of the tile
     bool ok = mbar_wait(done, 0, abort_flag);
@@ -357,17 +366,17 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem_base, FEW_MAX_ROWS);
+    tmem_dealloc(tmem_base, FEW_TILE_ROWS);
   }
   if (S > 1) cluster_sync();  // every CTA of the cluster has its sum in shared memory
   if (warp >= 2 && nt > 0 && !*abort_flag) {
     const int t0 = rank * nt / S, t1 = min((rank + 1) * nt / S, rows);
     const int et = threadIdx.x - 64;
     switch (S) {
-      case 1: few_finish<EPI, 1>(a, base, u, t0, t1, et, pos_s, seq_s); break;
-      case 2: few_finish<EPI, 2>(a, base, u, t0, t1, et, pos_s, seq_s); break;
-      case 4: few_finish<EPI, 4>(a, base, u, t0, t1, et, pos_s, seq_s); break;
-      case 8: few_finish<EPI, 8>(a, base, u, t0, t1, et, pos_s, seq_s); break;
+      case 1: few_finish<EPI, 1>(a, base, u, tok0, t0, t1, et, pos_s, seq_s); break;
+      case 2: few_finish<EPI, 2>(a, base, u, tok0, t0, t1, et, pos_s, seq_s); break;
+      case 4: few_finish<EPI, 4>(a, base, u, tok0, t0, t1, et, pos_s, seq_s); break;
+      case 8: few_finish<EPI, 8>(a, base, u, tok0, t0, t1, et, pos_s, seq_s); break;
     }
   }
   __syncwarp();
@@ -394,11 +403,13 @@ cudaError_t launch_few(const FewPlan& p, int* err, cudaStream_t stream) {
   FewArgs a;
   a.nkb = p.K / FW_BK;
   a.nt_max = p.nt_max;
+  a.units = p.units;
+  a.tiles = p.tiles;
   a.N = p.N;
   a.M = p.M;
   a.ep = p.ep;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.units * p.split);
+  cfg.gridDim = dim3(p.units * p.tiles * p.split);
   cfg.blockDim = dim3(FW_THREADS);
   cfg.dynamicSmemBytes = FW_SMEM;
   cfg.stream = stream;
@@ -417,8 +428,9 @@ cudaError_t launch_few(const FewPlan& p, int* err, cudaStream_t stream) {
 }  // namespace
 
 cudaError_t few_plan(FewPlan* p, const void* X, int M, int K, const void* W, int N, int epi, const FewEpi& ep,
-                     int num_sms, int nt_max) {
-  if (M <= 0 || N <= 0 || K <= 0 || K % FW_BK || (nt_max != 32 && nt_max != FEW_MAX_ROWS)) return cudaErrorInvalidValue;
+                     int num_sms, int rows) {
+  const int nt_max = rows <= 32 ? 32 : FEW_TILE_ROWS;
+  if (M <= 0 || N <= 0 || K <= 0 || K % FW_BK || rows <= 0) return cudaErrorInvalidValue;
   if ((reinterpret_cast<uintptr_t>(X) & 15) || (reinterpret_cast<uintptr_t>(W) & 15) ||
       (reinterpret_cast<uintptr_t>(ep.out) & 15) || ep.ldo % 4 || N % 4)
     return cudaErrorInvalidValue;
@@ -444,9 +456,15 @@ cudaError_t few_plan(FewPlan* p, const void* X, int M, int K, const void* W, int
   p->ep = ep;
   p->nt_max = nt_max;
   p->units = (N + FW_TILE - 1) / FW_TILE;
+  p->tiles = (rows + nt_max - 1) / nt_max;
   p->split = 1;
-  while (p->split < 8 && p->units * p->split * 2 <= 2 * num_sms && K / FW_BK / (p->split * 2) >= 1) p->split *= 2;
+  while (p->split < 8 && p->units * p->tiles * p->split * 2 <= 2 * num_sms && K / FW_BK / (p->split * 2) >= 1)
+    p->split *= 2;
   return cudaSuccess;
+}
+
+int few_rows(int N, int num_sms) {
+  return FEW_TILE_ROWS * std::max(1, 2 * num_sms / ((N + FW_TILE - 1) / FW_TILE));
 }
 
 cudaError_t few_launch(const FewPlan& p, int* err, cudaStream_t stream) {

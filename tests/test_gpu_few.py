@@ -65,6 +65,9 @@ STEPS = [
     (64, 128, 3, 2, 20),  # three blocks, 96 rows
     (64, 128, 1, 1, 40),  # suffix of 96 rows
     (64, 128, 1, 1, 5),   # suffix of 128 rows
+    (32, 97, 1, 0, 3),    # 129 rows: a second token tile of one row
+    (37, 90, 3, 0, 21),   # 381 rows of three ragged sequences
+    (64, 128, 8, 1, 5),   # suffixes of 128 rows, 1024 in all, after a refresh of 1536
 ]
 # heads of 64 and of 128 columns, grouped-query
 MODELS = {64: dict(d=768, H=12, G=4, F=1024), 128: dict(d=512, H=4, G=2, F=1536)}
