@@ -52,6 +52,64 @@ __device__ __forceinline__ void store_bf16x32(__nv_bfloat16* dst, const float* v
                        pack_bf16x2(v[8 * i + 4], v[8 * i + 5]), pack_bf16x2(v[8 * i + 6], v[8 * i + 7]));
 }
 
+// ------------------------------------------------------------------ softmax partials
+// A row's running softmax statistics over the columns seen so far: maximum m (= top-1 value),
+// its lowest column, the second largest value, sum of exp(z - m), and the entropy sum u = sum
+// exp(z - m) * y with y = (z - m) log2(e).
+struct RowStats {
+  float m = -INFINITY, s = 0.f, t2 = -INFINITY, u = 0.f;
+  int id = -1;
+};
+// 32 more columns, the first being col0 (columns from vocab on are ignored).  One thread holds
+// the row, so what bounds this is the length of its dependent chains: the two largest values
+// come from a tree, the sums run in four chains (column after column a 256-column tile took
+// about 10 us, the whole of a small model's LM head and the tail of a large one's).
+__device__ __forceinline__ void take_cols(RowStats& a, float (&v)[32], int col0, int vocab) {
+  if (col0 + 32 > vocab) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (col0 + i >= vocab) v[i] = -INFINITY;
+  }
+  float hi[16], lo[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    hi[i] = fmaxf(v[2 * i], v[2 * i + 1]);
+    lo[i] = fminf(v[2 * i], v[2 * i + 1]);
+  }
+#pragma unroll
+  for (int n = 8; n > 0; n >>= 1)
+#pragma unroll
+    for (int i = 0; i < n; ++i) {
+      lo[i] = max3f(fminf(hi[i], hi[i + n]), lo[i], lo[i + n]);
+      hi[i] = fmaxf(hi[i], hi[i + n]);
+    }
+  const float cm = hi[0];
+  if (cm > a.m) {
+#pragma unroll
+    for (int i = 31; i >= 0; --i)
+      if (v[i] == cm) a.id = col0 + i;  // the lowest of the chunk (columns arrive in increasing order)
+  }
+  a.t2 = fmaxf(fminf(cm, a.m), fmaxf(lo[0], a.t2));
+  const float m = fmaxf(a.m, cm);
+  if (m > -INFINITY) {
+    const float mb = m * kLog2e;
+    const float d = fmaf(a.m, kLog2e, -mb);  // -inf before the first live column
+    const float al = ex2_approx(d);
+    float u[4] = {a.s > 0.f ? al * fmaf(d, a.s, a.u) : 0.f, 0.f, 0.f, 0.f};
+    float s[4] = {a.s * al, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      const float y = fmaf(v[i], kLog2e, -mb);
+      const float e = ex2_approx(y);
+      s[i & 3] += e;
+      u[i & 3] = fmaf(e, fmaxf(y, -200.f), u[i & 3]);  // e = 0 below -126: the term's limit 0
+    }
+    a.s = (s[0] + s[1]) + (s[2] + s[3]);
+    a.u = (u[0] + u[1]) + (u[2] + u[3]);
+  }
+  a.m = m;
+}
+
 // ------------------------------------------------------------------ epilogues
 // (one-CTA tiles; the CTA-pair kernel has its own, staged through shared memory)
 struct Parts {};  // no earlier partial sums: one-CTA tiles are never split
@@ -152,56 +210,18 @@ __device__ __forceinline__ void epilogue_tile(uint32_t taddr, int row, int n_blk
       }
     }
   } else if constexpr (EPI == EPI_LMHEAD) {
-    // Online softmax over this tile's columns: running max m (= top-1 value), sum of
-    // exp(z - m), argmax (lowest column on ties: columns arrive in increasing order and
-    // only a strictly larger value replaces the leader), the second largest value, and
-    // the entropy sum u = sum exp(z - m) * y with y = (z - m) log2(e).
-    float m = -INFINITY, s = 0.f, t2 = -INFINITY, u = 0.f;
-    int id = -1;
+    RowStats a;  // online softmax over this tile's columns
 #pragma unroll 1
     for (int c = 0; c < BN; c += 32) {
       float v[32];
       load_cols(taddr, c, v, ps);
-      const int col0 = n0 + c;
-      float cm = m;
-      int cid = id;
-      float c2 = t2;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        if (col0 + i >= ep.vocab) v[i] = -INFINITY;
-        if (v[i] > cm) {
-          c2 = cm;
-          cm = v[i];
-          cid = col0 + i;
-        } else if (v[i] > c2) {
-          c2 = v[i];
-        }
-      }
-      if (cm > -INFINITY) {
-        const float mb = cm * kLog2e;
-        const float d = m * kLog2e - mb;  // -inf before the first live column
-        const float al = exp2f(d);
-        float acc = s * al;
-        float accu = s > 0.f ? al * fmaf(d, s, u) : 0.f;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float y = fmaf(v[i], kLog2e, -mb);
-          const float e = exp2f(y);
-          acc += e;
-          accu = fmaf(e, fmaxf(y, -200.f), accu);  // e = 0 below -149: the term's limit 0
-        }
-        s = acc;
-        u = accu;
-      }
-      m = cm;
-      id = cid;
-      t2 = c2;
+      take_cols(a, v, n0 + c, ep.vocab);
     }
     if (live) {
       const int nblk = (N + BN - 1) / BN;
       float4* part = reinterpret_cast<float4*>(ep.out);
-      part[(size_t)row * nblk + n_blk] = make_float4(m, s, __int_as_float(id), t2);
-      if (ep.ent_part) ep.ent_part[(size_t)row * nblk + n_blk] = u;
+      part[(size_t)row * nblk + n_blk] = make_float4(a.m, a.s, __int_as_float(a.id), a.t2);
+      if (ep.ent_part) ep.ent_part[(size_t)row * nblk + n_blk] = a.u;
     }
   }
 }
@@ -762,53 +782,18 @@ __device__ __forceinline__ void epilogue_pair(const Src& s, Stage& o, const CUte
       o.issue(tmc, b, n_blk * 128 + piece * G2 + c, o.row0, false);
     }
   } else if constexpr (EPI == EPI_LMHEAD) {
-    // Online softmax over this tile's columns (see epilogue_tile); one float4 per row.
-    float m = -INFINITY, sum = 0.f, t2 = -INFINITY, u = 0.f;
-    int id = -1;
+    RowStats a;  // online softmax over this tile's columns; one float4 per row
 #pragma unroll 1
     for (int c = 0; c < 256; c += 32) {
       float v[32];
       src_cols(s, c, v);
-      const int col0 = n0 + c;
-      float cm = m;
-      int cid = id;
-      float c2 = t2;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        if (col0 + i >= ep.vocab) v[i] = -INFINITY;
-        if (v[i] > cm) {
-          c2 = cm;
-          cm = v[i];
-          cid = col0 + i;
-        } else if (v[i] > c2) {
-          c2 = v[i];
-        }
-      }
-      if (cm > -INFINITY) {
-        const float mb = cm * kLog2e;
-        const float d = m * kLog2e - mb;  // -inf before the first live column
-        const float al = exp2f(d);
-        float acc = sum * al;
-        float accu = sum > 0.f ? al * fmaf(d, sum, u) : 0.f;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float y = fmaf(v[i], kLog2e, -mb);
-          const float e = exp2f(y);
-          acc += e;
-          accu = fmaf(e, fmaxf(y, -200.f), accu);  // e = 0 below -149: the term's limit 0
-        }
-        sum = acc;
-        u = accu;
-      }
-      m = cm;
-      id = cid;
-      t2 = c2;
+      take_cols(a, v, n0 + c, ep.vocab);
     }
     if (row < M) {
       const int nblk = (N + 255) / 256;
       float4* part = reinterpret_cast<float4*>(ep.out);
-      part[(size_t)row * nblk + n_blk] = make_float4(m, sum, __int_as_float(id), t2);
-      if (ep.ent_part) ep.ent_part[(size_t)row * nblk + n_blk] = u;
+      part[(size_t)row * nblk + n_blk] = make_float4(a.m, a.s, __int_as_float(a.id), a.t2);
+      if (ep.ent_part) ep.ent_part[(size_t)row * nblk + n_blk] = a.u;
     }
   }
 }
@@ -1701,7 +1686,12 @@ cudaError_t gemm_plan(GemmPlan* plan, const void* A, int M, int K, const void* W
       splits = forced_splits > 0 ? forced_splits : split_auto;
     }
   } else if (bn == 0) {
-    if (M > BM && pairs >= 1) {
+    // (the LM head of at most 128 rows is a weight stream whose tiles all take the same time:
+    // whichever form leaves less of its last round empty, V = 126464: 494 tiles on 152 SMs or on
+    // 76 pairs, 175 us against 160)
+    const bool pair_fuller = epi == EPI_LMHEAD && pairs >= 1 &&
+                             wave_efficiency(pair_tiles, pairs) > wave_efficiency(pair_tiles, num_sms);
+    if ((M > BM && pairs >= 1) || pair_fuller) {
       bn = 256;
       cg = 2;
       splits = split_auto;
