@@ -215,26 +215,30 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   const int jb = split ? rank * nb / S : 0, n = (split ? (rank + 1) * nb / S : nb) - jb;  // its key blocks
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------ TMA producer
-      bool ok = true;
-      int stage = 0;
-      uint32_t phase = 0;
-      long issued = 0;
+    // ------------------------------------------------ TMA producer (the whole warp, one lane issues)
+    const bool leader = elect_one();
+    bool ok = true;
+    int stage = 0;
+    uint32_t phase = 0;
+    int issued = 0;
+    if (leader) {
       mbar_arrive_expect_tx(q_full, live * 32 * HD * 2);
       for (int i = 0; i < live; ++i) {
         const int h = g * rep + (band0 + i) / nch, r0 = q_off + 32 * ((band0 + i) % nch);
         const uint32_t dst = sQ + (i >> 2) * C::Q_BYTES + (i & 3) * (32 * 128);
         for (int bx = 0; bx < C::KB; ++bx) tma_load_2d(dst + bx * AT_BOX, &tq, h * HD + bx * 64, r0, q_full);
       }
-      // consumption order: K_0, then per block K_{j+1}, V_j
-      for (int u = 0; u < 2 * n; ++u) {
-        const bool is_v = u == 2 * n - 1 || (u > 0 && (u & 1) == 0);
-        const int j = jb + (is_v ? (u - 1) >> 1 : (u + 1) >> 1);
-        if (!mbar_wait(kv_empty0 + 8 * stage, phase ^ 1u, abort_flag)) {
-          ok = false;
-          break;
-        }
+    }
+    __syncwarp();
+    // consumption order: K_0, then per block K_{j+1}, V_j
+    for (int u = 0; u < 2 * n; ++u) {
+      const bool is_v = u == 2 * n - 1 || (u > 0 && (u & 1) == 0);
+      const int j = jb + (is_v ? (u - 1) >> 1 : (u + 1) >> 1);
+      if (!__all_sync(0xffffffffu, mbar_wait_inline(kv_empty0 + 8 * stage, phase ^ 1u, abort_flag))) {
+        ok = false;
+        break;
+      }
+      if (leader) {
         const uint32_t dst = sKV + stage * C::STAGE_BYTES, bar = kv_full0 + 8 * stage;
         mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
         if (!is_v) {
@@ -243,22 +247,23 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         } else {
           for (int bx = 0; bx < 2; ++bx) tma_load_3d(dst + bx * C::VBOX, &tv, j * 128 + bx * 64, 0, b * G + g, bar);
         }
-        ++issued;
-        if (++stage == C::STAGES) {
-          stage = 0;
-          phase ^= 1u;
-        }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
-        // wait (bounded) for the copies this thread issued before leaving
-        volatile int no_abort = 0;
-        mbar_wait(q_full, 0, &no_abort);
-        for (int s = 0; s < C::STAGES && s < issued; ++s) {
-          const long arms = (issued - 1 - s) / C::STAGES + 1;
-          mbar_wait(kv_full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
-        }
+      __syncwarp();
+      ++issued;
+      if (++stage == C::STAGES) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    }
+    if (!ok) {
+      *abort_flag = 1;
+      if (leader) report_error(err, DERR_WAIT_TIMEOUT);
+      // wait (bounded) for the copies issued before leaving
+      volatile int no_abort = 0;
+      mbar_wait(q_full, 0, &no_abort);
+      for (int s = 0; s < C::STAGES && s < issued; ++s) {
+        const int arms = (issued - 1 - s) / C::STAGES + 1;
+        mbar_wait(kv_full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
       }
     }
   } else if (warp == 1) {

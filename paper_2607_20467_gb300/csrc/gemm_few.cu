@@ -246,11 +246,11 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
     }
   };
   // the first stages' weights, before the dependent-launch wait (no kernel of the step writes them)
-  int pre = 0;
-  if (a.ep.w_early && threadIdx.x == 0)
-    for (; pre < stages && pre < nkb; ++pre) {
-      mbar_expect_tx(full0 + 8 * pre, FW_W_BYTES);
-      load_w(pre, pre);
+  const int pre = a.ep.w_early ? min(stages, nkb) : 0;
+  if (threadIdx.x == 0)
+    for (int kb = 0; kb < pre; ++kb) {
+      mbar_expect_tx(full0 + 8 * kb, FW_W_BYTES);
+      load_w(kb, kb);
     }
   if (warp == 1) tmem_alloc(holder, FEW_TILE_ROWS);
   tc_fence_before();
@@ -269,34 +269,40 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   }
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------ TMA producer
-      bool ok = true;
-      int issued = 0;
-      for (int kb = 0; kb < (nt > 0 ? nkb : pre); ++kb) {
-        const int stage = kb % stages;
-        const bool have_w = kb < pre;
-        if (!have_w && !mbar_wait(empty0 + 8 * stage, ((uint32_t)(kb / stages) & 1u) ^ 1u, abort_flag)) {
-          ok = false;
-          break;
-        }
+    // ------------------------------------------------ TMA producer (the whole warp, one lane issues)
+    const bool leader = elect_one();
+    bool ok = true;
+    int issued = 0, stage = 0;
+    uint32_t phase = 0;
+    for (int kb = 0; kb < (nt > 0 ? nkb : pre); ++kb) {
+      const bool have_w = kb < pre;
+      if (!have_w && !__all_sync(0xffffffffu, mbar_wait_inline(empty0 + 8 * stage, phase ^ 1u, abort_flag))) {
+        ok = false;
+        break;
+      }
+      if (leader) {
         mbar_arrive_expect_tx(full0 + 8 * stage, (have_w ? 0 : FW_W_BYTES) + nt * 128);
         if (!have_w) load_w(stage, kb);
         for (int b = 0; b < nt / 32; ++b)
           tma_load_2d(base + (uint32_t)(stage * stage_bytes + FW_W_BYTES + b * FW_XBOX_BYTES), &tx, (kb0 + kb) * FW_BK,
                       tok0 + b * 32, full0 + 8 * stage);
-        ++issued;
       }
-      if (!ok) {
-        *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
+      __syncwarp();
+      ++issued;
+      if (++stage == stages) {
+        stage = 0;
+        phase ^= 1u;
       }
-      if (!ok || nt == 0) {  // every copy issued lands before the CTA leaves (bounded)
-        for (int s = 0; s < stages && s < issued; ++s) {
-          const int arms = (issued - 1 - s) / stages + 1;
-          volatile int no_abort = 0;
-          mbar_wait(full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
-        }
+    }
+    if (!ok) {
+      *abort_flag = 1;
+      if (leader) report_error(err, DERR_WAIT_TIMEOUT);
+    }
+    if (!ok || nt == 0) {  // every copy issued lands before the CTA leaves (bounded)
+      for (int s = 0; s < stages && s < issued; ++s) {
+        const int arms = (issued - 1 - s) / stages + 1;
+        volatile int no_abort = 0;
+        mbar_wait(full0 + 8 * s, (uint32_t)((arms - 1) & 1), &no_abort);
       }
     }
   } else if (warp == 1) {

@@ -1170,68 +1170,78 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------ TMA producer (both CTAs)
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      Item it;
-      for (int idx = 0; ok && next_item(idx, sc, cluster, it); ++idx) {
-        int m_blk, n_blk;
-        tile_mn(it.t, m_blk, n_blk);
-        const int kb0 = it.ku0 * KA2, kb1 = it.ku1 * KA2;
-        // this CTA's half of the weight rows of the item: 128 rows of a whole tile, or 64
-        // of a half-width piece (SwiGLU: the gate rows in the leader, the matching up rows
-        // in the peer, as for whole tiles)
-        const bool hw = it.width != 256;
-        const int wrow = n_blk * 256 +
-                         (!hw ? (int)rank * 128
-                              : (EPI == EPI_SWIGLU ? (int)rank * 128 + it.piece * 64 : it.piece * 128 + (int)rank * 64));
-        const CUtensorMap* tw_map = hw ? &tmbh : &tmb;
-        const CUtensorMap* ta_map = &tma;
-        if (FUSE && it.g == 1) {
-          // the second GEMM reads act columns [ku0 * 64, ku1 * 64) of rows m_blk: wait until
-          // the first GEMM's tiles writing them (act columns 128 n .. 128 n + 127 from tile n,
-          // both CTAs of its pair) have stored them
-          ta_map = &ta2;
-          tw_map = &tb2;
-          const int need = 2 * ((it.ku1 + 1) / 2 - it.ku0 / 2);
-          int* dep = f_dep + m_blk * splits2 + it.sp;
-          if (!wait_flag_geq(dep, need, abort_flag)) {
-            ok = false;
-            break;
-          }
-          fence_proxy_async_global();  // the act stores (acquired) before this CTA's TMA loads
-          // the last of the pair CTAs that wait on this counter resets it for the next launch
-          if (atomicAdd(f_pass + m_blk * splits2 + it.sp, 1) == 2 * num_n2 - 1) {
-            atomicExch(dep, 0);
-            atomicExch(f_pass + m_blk * splits2 + it.sp, 0);
+    // ------------------------------------------------ TMA producer (both CTAs; the whole warp,
+    // one lane issues: see elect_one)
+    const bool leader = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    Item it;
+    for (int idx = 0; ok && next_item(idx, sc, cluster, it); ++idx) {
+      int m_blk, n_blk;
+      tile_mn(it.t, m_blk, n_blk);
+      const int kb0 = it.ku0 * KA2, kb1 = it.ku1 * KA2;
+      // this CTA's half of the weight rows of the item: 128 rows of a whole tile, or 64
+      // of a half-width piece (SwiGLU: the gate rows in the leader, the matching up rows
+      // in the peer, as for whole tiles)
+      const bool hw = it.width != 256;
+      const int wrow = n_blk * 256 +
+                       (!hw ? (int)rank * 128
+                            : (EPI == EPI_SWIGLU ? (int)rank * 128 + it.piece * 64 : it.piece * 128 + (int)rank * 64));
+      const CUtensorMap* tw_map = hw ? &tmbh : &tmb;
+      const CUtensorMap* ta_map = &tma;
+      if (FUSE && it.g == 1) {
+        // the second GEMM reads act columns [ku0 * 64, ku1 * 64) of rows m_blk: wait until
+        // the first GEMM's tiles writing them (act columns 128 n .. 128 n + 127 from tile n,
+        // both CTAs of its pair) have stored them
+        ta_map = &ta2;
+        tw_map = &tb2;
+        const int need = 2 * ((it.ku1 + 1) / 2 - it.ku0 / 2);
+        int* dep = f_dep + m_blk * splits2 + it.sp;
+        bool there = true;
+        if (leader) {
+          there = wait_flag_geq(dep, need, abort_flag);
+          if (there) {
+            fence_proxy_async_global();  // the act stores (acquired) before this CTA's TMA loads
+            // the last of the pair CTAs that wait on this counter resets it for the next launch
+            if (atomicAdd(f_pass + m_blk * splits2 + it.sp, 1) == 2 * num_n2 - 1) {
+              atomicExch(dep, 0);
+              atomicExch(f_pass + m_blk * splits2 + it.sp, 0);
+            }
           }
         }
-        const uint32_t stage_tx = 2u * (uint32_t)(hw ? A2_STAGE_BYTES + B2_STAGE_BYTES / 2 : STAGE2_BYTES);
-        for (int kb = kb0; kb < kb1; kb += KA2) {
-          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1u, abort_flag)) {
-            ok = false;
-            break;
-          }
+        if (!__all_sync(0xffffffffu, there)) {
+          ok = false;
+          break;
+        }
+      }
+      const uint32_t stage_tx = 2u * (uint32_t)(hw ? A2_STAGE_BYTES + B2_STAGE_BYTES / 2 : STAGE2_BYTES);
+      for (int kb = kb0; kb < kb1; kb += KA2) {
+        if (!__all_sync(0xffffffffu, mbar_wait_inline(empty0 + 8 * stage, phase ^ 1u, abort_flag))) {
+          ok = false;
+          break;
+        }
+        if (leader) {
           const uint32_t full_leader = mapa_shared(full0 + 8 * stage, lead);
           if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * stage, stage_tx);
+#pragma unroll
           for (int a = 0; a < KA2; ++a) {
             tma_load_2d_pair(sA + stage * A2_STAGE_BYTES + a * A_STAGE_BYTES, ta_map, (kb + a) * BK,
                              m_blk * 256 + (int)rank * 128, full_leader);
             tma_load_2d_pair(sB + stage * B2_STAGE_BYTES + a * B2_BLOCK_BYTES, tw_map, (kb + a) * BK, wrow,
                              full_leader);
           }
-          if (++stage == STAGES2) {
-            stage = 0;
-            phase ^= 1u;
-          }
+        }
+        __syncwarp();
+        if (++stage == STAGES2) {
+          stage = 0;
+          phase ^= 1u;
         }
       }
-      if (!ok) {
-        *abort_flag = 1;
-        report_error(err, DERR_WAIT_TIMEOUT);
-      }
+    }
+    if (!ok) {
+      *abort_flag = 1;
+      if (leader) report_error(err, DERR_WAIT_TIMEOUT);
     }
   } else if (warp == 1) {
     if (rank == 0) {
