@@ -7,8 +7,8 @@
 // MMA time of 256 (18 us per 256 x 256 x 4096 tile) on as many SM pairs as there are column
 // tiles (48 of 76 for QKV, 16 for O).  Here the operands are swapped: 128 weight rows on the
 // M side, the tokens (rounded up to 32) on the N side, so the MMA time follows the tokens, and
-// each tile of 128 weight rows is split by K over a cluster of S CTAs.  S is the largest power
-// of two up to 8 that leaves a CTA a K block and the grid within two CTAs per SM.
+// each tile of 128 weight rows is split by K over a cluster of S CTAs, as far as the grid stays
+// within two CTAs per SM and the shares are worth it (few_plan).
 //
 // One CTA = one tile's share of K (192 threads: TMA producer, MMA issuer, four epilogue
 // warps).  Its fp32 sum goes from TMEM to its idle operand ring; after a cluster barrier each
@@ -463,9 +463,16 @@ cudaError_t few_plan(FewPlan* p, const void* X, int M, int K, const void* W, int
   p->nt_max = nt_max;
   p->units = (N + FW_TILE - 1) / FW_TILE;
   p->tiles = (rows + nt_max - 1) / nt_max;
+  // (at least this many K blocks for each CTA of a split: the cluster's barrier and its reads of
+  // distributed shared memory cost more than a shorter share saves.  d 768, ffn 2048, 384 rows,
+  // four layers: 222 us a step with splits down to one block, 206 with two and 196 so; a long K
+  // is a weight stream, which wants all eight)
+  const int nkb = K / FW_BK;
+  auto fits = [&](int S) {
+    return p->units * p->tiles * S <= 2 * num_sms && nkb / S >= (S == 2 ? 2 : S == 4 ? 3 : 8);
+  };
   p->split = 1;
-  while (p->split < 8 && p->units * p->tiles * p->split * 2 <= 2 * num_sms && K / FW_BK / (p->split * 2) >= 1)
-    p->split *= 2;
+  while (p->split < 8 && fits(2 * p->split)) p->split *= 2;
   return cudaSuccess;
 }
 
