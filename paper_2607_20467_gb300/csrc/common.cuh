@@ -299,10 +299,11 @@ struct DcvParams {
 // N + i).  With ent, jpde[b] accumulates Eq. entropy_bound of the set row b commits.
 // cmt: committed flags [batch][N + M] (read and written with acceptance 1 only).
 // kcap (may be NULL): per-row cap on K (RowPlan::kcap).
+// all_done (pinned host memory): set to 1 by the row that is the last to finish.
 cudaError_t dcv_commit_launch(int32_t* x, int32_t* p, int32_t* k_out, int32_t* steps,
                               const int32_t* ids, const float* c, const float* ent, float* jpde, int batch,
-                              int N, int M, const DcvParams& prm, int32_t* done_count, uint8_t* cmt,
-                              const int* kcap, cudaStream_t stream);
+                              int N, int M, const DcvParams& prm, int32_t* done_count, int32_t* all_done,
+                              uint8_t* cmt, const int* kcap, cudaStream_t stream);
 // Block acceptance from bf16 logits (dcl_accept), in two passes: the softmax statistics of
 // every uncommitted position in accept_chunks(B * P, V) chunks of its row, partials to part
 // [B * P][chunks] ({max, sum exp(z - max), id, entropy sum}), then their merge into ids and c1

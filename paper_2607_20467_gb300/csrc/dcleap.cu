@@ -105,10 +105,11 @@ struct dcl_ctx {
   bool profiling = false;
   ProfGraph prof[STEP_BRANCHES];  // profiling: one graph per branch, the host takes the step's
   int prof_last = -1;             // the branch of the last profiled step
-  // pinned: h_done [2], the error word's copy, and a buffer for the copies of the state and of
+  // pinned: h_done, the error word's copy, and a buffer for the copies of the state and of
   // the results (a copy from or to pageable memory waits for the stream each time)
   int32_t* h_done = nullptr;
   int32_t* h_err = nullptr;
+  int32_t* h_all = nullptr;  // set by the device when every row has finished
   int32_t* h_buf = nullptr;
   // scratch of the single-kernel entry points, kept from call to call up to OP_SCRATCH_KEEP
   void* op_buf = nullptr;
@@ -361,7 +362,7 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
                   c->dcfg.contiguous_drafts, c->dcfg.acceptance, c->dcfg.block_len};
     q.begin(DCL_K_DCV);
     q.end(dcv_commit_launch(c->x, c->p, c->k, c->steps, c->top1, co.conf, c->ent, c->jpde, c->B, c->N, c->M, prm,
-                            c->done_count, c->cmt, c->rp.kcap, c->stream),
+                            c->done_count, c->h_all, c->cmt, c->rp.kcap, c->stream),
           "dcv_commit");
   }
 }
@@ -931,6 +932,7 @@ dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t ma
     return fail(nullptr, DCL_ERR_CUDA, "pinned host buffer / event creation failed");
   }
   c->h_err = c->h_done + 2;
+  c->h_all = c->h_done + 3;
   c->h_buf = c->h_done + PINNED_HEAD;
   *out = c;
   return DCL_OK;
@@ -1081,16 +1083,19 @@ dcl_status dcl_generate(dcl_ctx* c, int32_t max_steps, int32_t* out, dcl_stats* 
   CUDA_TRY(c, cudaMemcpyAsync(&c->h_done[0], c->done_count, 4, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   done = c->h_done[0] >= c->B;
+  // the step that finishes the last row says so in host memory itself (a copy of the count
+  // after each step stood between the step graphs); an event orders the read
+  volatile int32_t* const all = c->h_all;
+  *all = 0;
   while (!done && launched < max_steps) {
     const dcl_status ls = launch_step(c);
     if (ls != DCL_OK) return ls;
     const int slot = launched & 1;
-    CUDA_TRY(c, cudaMemcpyAsync(&c->h_done[slot], c->done_count, 4, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaEventRecord(c->ev_done[slot], c->stream));
     ++launched;
     if (launched >= 2) {
       CUDA_TRY(c, cudaEventSynchronize(c->ev_done[slot ^ 1]));
-      if (c->h_done[slot ^ 1] >= c->B) done = true;
+      done = *all != 0;
     }
   }
   // the results in one wait: p, steps and the entropy bound of every row, then its tokens
@@ -1105,7 +1110,7 @@ dcl_status dcl_generate(dcl_ctx* c, int32_t max_steps, int32_t* out, dcl_stats* 
     CUDA_TRY(c, cudaMemcpy2DAsync(xh, 4 * (size_t)c->M, c->x + c->N, 4 * (size_t)c->T, 4 * (size_t)c->M, c->B,
                                   cudaMemcpyDeviceToHost, c->stream));
   dcl_status s = check_device(c);
-  if (launched > 0 && c->h_done[(launched - 1) & 1] >= c->B) done = true;
+  done = done || *all != 0;
   if (s != DCL_OK) return s;
   if (out) memcpy(out, xh, 4 * (size_t)c->B * c->M);
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();

@@ -367,8 +367,8 @@ __global__ void dcv_commit_kernel(int32_t* __restrict__ x, int32_t* __restrict__
                                   int32_t* __restrict__ k_out, int32_t* __restrict__ steps,
                                   const int32_t* __restrict__ ids, const float* __restrict__ c,
                                   const float* __restrict__ ent, float* __restrict__ jpde, int N, int M,
-                                  DcvParams prm, int32_t* done_count, uint8_t* __restrict__ cmt,
-                                  const int* __restrict__ kcap) {
+                                  DcvParams prm, int32_t* done_count, volatile int32_t* all_done,
+                                  uint8_t* __restrict__ cmt, const int* __restrict__ kcap) {
   pdl_wait();
   pdl_launch_dependents();
   const int b = blockIdx.x;
@@ -400,7 +400,7 @@ __global__ void dcv_commit_kernel(int32_t* __restrict__ x, int32_t* __restrict__
       k_out[b] = K;
       p[b] = np;
       steps[b] += 1;
-      if (np >= T) atomicAdd(done_count, 1);
+      if (np >= T && atomicAdd(done_count, 1) + 1 == (int)gridDim.x) *all_done = 1;
     }
     return;
   }
@@ -426,7 +426,7 @@ __global__ void dcv_commit_kernel(int32_t* __restrict__ x, int32_t* __restrict__
     k_out[b] = K;
     p[b] = pb + K;
     steps[b] += 1;
-    if (pb + K >= T) atomicAdd(done_count, 1);
+    if (pb + K >= T && atomicAdd(done_count, 1) + 1 == (int)gridDim.x) *all_done = 1;
   }
 }
 
@@ -762,11 +762,11 @@ cudaError_t lmhead_combine_launch(const float4* part, const float* upart, int ro
 
 cudaError_t dcv_commit_launch(int32_t* x, int32_t* p, int32_t* k_out, int32_t* steps,
                               const int32_t* ids, const float* c, const float* ent, float* jpde, int batch,
-                              int N, int M, const DcvParams& prm, int32_t* done_count, uint8_t* cmt,
-                              const int* kcap, cudaStream_t stream) {
+                              int N, int M, const DcvParams& prm, int32_t* done_count, int32_t* all_done,
+                              uint8_t* cmt, const int* kcap, cudaStream_t stream) {
   if (prm.acceptance == 1 && (prm.block_len < 1 || !cmt)) return cudaErrorInvalidValue;
   return launch_pdl(dcv_commit_kernel, batch, 32, 0, stream, x, p, k_out, steps, ids, c, ent, jpde, N, M, prm,
-                    done_count, cmt, kcap);
+                    done_count, all_done, cmt, kcap);
 }
 
 int accept_chunks(int n, int V) {
