@@ -202,6 +202,32 @@ cudaError_t few_plan(FewPlan* plan, const void* X, int M, int K, const void* W, 
 int few_rows(int N, int num_sms);
 cudaError_t few_launch(const FewPlan& plan, int* err, cudaStream_t stream);
 
+// ---------------------------------------------------------------- mid-row GEMM (gemm_mid.cu)
+// The same with CTA pairs, 256 weight rows (N a multiple of 256) by tiles of up to 256 rows of X;
+// epilogues EPI_RESID_F32, EPI_QKV_ROPE, EPI_SWIGLU.
+struct MidShape {   // how `rows` rows are cut: tiles of tokens, splits of K, estimated time in K
+  int tt = 0, splits = 1;  // blocks of a 256 x 256 tile
+  double cost = 0;
+};
+MidShape mid_shape(int rows, int N, int K, int epi, int pairs);
+struct MidTokens {  // X in boxes of 16, 32, .. 128 rows
+  CUtensorMap box[8];
+};
+struct MidPlan {
+  CUtensorMap tw;
+  MidTokens tx;
+  int M = 0, N = 0, K = 0, epi = EPI_RESID_F32;
+  FewEpi ep;
+  int grid = 0;
+  int shape = 0;                     // of M rows: tt + 256 * splits
+  const uint16_t* shapes = nullptr;  // device, by rows / 32 (with ep.m_dev)
+  size_t flags_needed = 0;           // ints of zero-initialised counters
+  int* flags = nullptr;
+};
+cudaError_t mid_plan(MidPlan* plan, const void* X, int M, int K, const void* W, int N, int epi, const FewEpi& ep,
+                     int num_sms);
+cudaError_t mid_launch(const MidPlan& plan, int* err, cudaStream_t stream);
+
 // ---------------------------------------------------------------- attention (attention_tc.cu)
 // softmax(q k^T / sqrt(hd)) v per (sequence, head): the query rows of sequence b are rows
 // [seq_off[b], seq_off[b] + seq_len[b]) of qkv (q columns) and of out (NULL tables: b*T and
@@ -258,16 +284,12 @@ struct RowPlan {
 // current block).  update = 0 plans the rows without recording the prefix end (a forward
 // that commits nothing, e.g. a debug pass, leaves the next step's refresh decision
 // unchanged).
-// select: the conditional node that takes the step's branch (StepBranch of the row count), or 0.
+// select: the conditional node that takes the step's branch (branches[rows / 32], rounded up), or 0.
 cudaError_t row_plan_launch(const RowPlan& rp, const int32_t* p, int batch, int N, int T, int block_len,
                             int cached, int update, int32_t* x, int window, int mask_id,
-                            cudaGraphConditionalHandle select, int few_max, cudaStream_t stream);
-// The GEMM kernels of a step, by the rows it computes (few_max: the most that the shape's
-// few-row GEMMs take).
-enum StepBranch : int { STEP_PAIR = 0, STEP_FEW32 = 1, STEP_FEW = 2, STEP_BRANCHES = 3 };
-__host__ __device__ inline int step_branch(int rows, int few_max) {
-  return rows <= 32 ? STEP_FEW32 : rows <= few_max ? STEP_FEW : STEP_PAIR;
-}
+                            cudaGraphConditionalHandle select, const uint16_t* branches, cudaStream_t stream);
+// The GEMM kernels of a step, by the rows it computes.
+enum StepBranch : int { STEP_PAIR = 0, STEP_FEW32 = 1, STEP_FEW = 2, STEP_MID = 3, STEP_BRANCHES = 4 };
 cudaError_t embed_remask_launch(int32_t* x, const int32_t* p, int batch, int T, int window,
                                 int mask_id, int vocab, const __nv_bfloat16* embed, int d,
                                 float* h, int* err, const RowPlan& rp, cudaStream_t stream);

@@ -101,6 +101,12 @@ struct dcl_ctx {
   // [1] for up to few_max; empty where no step of this shape takes them
   std::vector<FewPlan> few[2];
   int few_max = 0;
+  // the mid-row GEMMs (4 per layer; empty where the shape does not allow them).  By rows / 32
+  // rounded up: the step's branch, then the tiling of each of the four (the same on the device)
+  std::vector<MidPlan> mid;
+  std::vector<uint16_t> row_tab;
+  uint16_t* row_tab_dev = nullptr;
+  size_t row_tab_n = 0;
   cudaGraphExec_t gexec = nullptr;
   bool profiling = false;
   ProfGraph prof[STEP_BRANCHES];  // profiling: one graph per branch, the host takes the step's
@@ -273,7 +279,7 @@ struct Enq {
 void enqueue_rows(dcl_ctx* c, Enq& q, bool update, cudaGraphConditionalHandle select) {
   q.begin(DCL_K_ROWPLAN);
   q.end(row_plan_launch(c->rp, c->p, c->B, c->N, c->T, c->dcfg.block_len, c->dcfg.kv_cache, update ? 1 : 0, c->x,
-                        c->dcfg.acceptance ? 0 : c->window, c->cfg.mask_id, select, c->few_max, c->stream),
+                        c->dcfg.acceptance ? 0 : c->window, c->cfg.mask_id, select, c->row_tab_dev, c->stream),
         "row_plan");
 }
 
@@ -285,7 +291,8 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
   const dcl_model_config& m = c->cfg;
   const int R = c->B * c->T;
   const int d = m.d_model;
-  const std::vector<FewPlan>* few = branch == STEP_PAIR ? nullptr : &c->few[branch == STEP_FEW32 ? 0 : 1];
+  const std::vector<FewPlan>* few =
+      branch == STEP_FEW32 || branch == STEP_FEW ? &c->few[branch == STEP_FEW32 ? 0 : 1] : nullptr;
   const int rows = std::min(R, branch == STEP_FEW32 ? 32 : branch == STEP_FEW ? c->few_max : R);  // at most
   AttnRows ar;  // the attention's query rows: every position, or as the row plan says
   ar.most = std::min(c->T, rows);
@@ -310,11 +317,17 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
     const Layer& L = c->layers[l];
     const GemmPlan* P = &c->plans[4 * l];
     const FewPlan* F = few ? &(*few)[4 * l] : nullptr;
+    const MidPlan* Q = branch == STEP_MID ? &c->mid[4 * l] : nullptr;
+    auto gemm = [&](int i) {
+      return F ? few_launch(F[i], c->derr, c->stream)
+             : Q ? mid_launch(Q[i], c->derr, c->stream)
+                 : gemm_launch(P[i], c->derr, c->stream);
+    };
     q.begin(DCL_K_RMSNORM);
     q.end(rmsnorm_launch(c->h, L.attn_norm, c->xn, rows, d, m.rms_eps, c->rp.counts, nullptr, F != nullptr, c->stream),
           "rmsnorm");
     q.begin(DCL_K_GEMM_QKV);
-    q.end(F ? few_launch(F[0], c->derr, c->stream) : gemm_launch(P[0], c->derr, c->stream), "gemm_qkv");
+    q.end(gemm(0), "gemm_qkv");
     if (!c->kv_fused) {
       q.begin(DCL_K_VTRANSPOSE);
       q.end(attention_transpose_launch(c->attn_plans[l], c->stream), "v_transpose");
@@ -322,18 +335,18 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
     q.begin(DCL_K_ATTENTION);
     q.end(attention_core_launch(c->attn_plans[l], ar, c->derr, c->stream), "attention");
     q.begin(DCL_K_GEMM_O);
-    q.end(F ? few_launch(F[1], c->derr, c->stream) : gemm_launch(P[1], c->derr, c->stream), "gemm_o");
+    q.end(gemm(1), "gemm_o");
     q.begin(DCL_K_RMSNORM);
     q.end(rmsnorm_launch(c->h, L.mlp_norm, c->xn, rows, d, m.rms_eps, c->rp.counts, nullptr, F != nullptr, c->stream),
           "rmsnorm");
-    if (!F && P[2].fuse) {  // gate/up + SwiGLU and down + residual in one launch
+    if (!F && !Q && P[2].fuse) {  // gate/up + SwiGLU and down + residual in one launch
       q.begin(DCL_K_GEMM_MLP);
       q.end(gemm_launch(P[2], c->derr, c->stream), "gemm_mlp");
     } else {
       q.begin(DCL_K_GEMM_GATEUP);
-      q.end(F ? few_launch(F[2], c->derr, c->stream) : gemm_launch(P[2], c->derr, c->stream), "gemm_gateup");
+      q.end(gemm(2), "gemm_gateup");
       q.begin(DCL_K_GEMM_DOWN);
-      q.end(F ? few_launch(F[3], c->derr, c->stream) : gemm_launch(P[3], c->derr, c->stream), "gemm_down");
+      q.end(gemm(3), "gemm_down");
     }
     if (snapshots && q.err == cudaSuccess)
       q.err = cudaMemcpyAsync(c->snap + (size_t)(l + 1) * R * d, c->h, sizeof(float) * R * d,
@@ -367,13 +380,13 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
   }
 }
 
+int branch_of(const dcl_ctx* c, int rows) { return c->row_tab[(size_t)(rows + 31) >> 5]; }
+
 // The branch of the next step: by its rows, as the row plan counts them.  Fixed by the shape
 // without a key / value cache; else read from the device (synchronises).
 dcl_status current_branch(dcl_ctx* c, int* out) {
-  *out = STEP_PAIR;
-  if (c->few[0].empty()) return DCL_OK;
   if (!c->dcfg.kv_cache) {
-    *out = step_branch(c->B * c->T, c->few_max);
+    *out = branch_of(c, c->B * c->T);
     return DCL_OK;
   }
   int32_t* const ph = c->h_buf;
@@ -390,7 +403,7 @@ dcl_status current_branch(dcl_ctx* c, int* out) {
     const int start = fresh ? end : 0;
     rows += (c->dcfg.kv_cache == 2 && start != 0 ? std::min(end + Bk, c->T) : c->T) - start;
   }
-  *out = step_branch((int)rows, c->few_max);
+  *out = branch_of(c, (int)rows);
   return DCL_OK;
 }
 
@@ -419,6 +432,13 @@ dcl_status capture_into(dcl_ctx* c, cudaGraph_t g, ProfGraph* prof, Body body) {
   return DCL_OK;
 }
 
+// Does a step of this context take the branch?  (Without a key / value cache its rows are fixed.)
+bool has_branch(const dcl_ctx* c, int br) {
+  if (!c->dcfg.kv_cache) return branch_of(c, c->B * c->T) == br;
+  const size_t n = (size_t)(c->B * c->T + 31) / 32 + 1;
+  return std::find(c->row_tab.begin(), c->row_tab.begin() + n, (uint16_t)br) != c->row_tab.begin() + n;
+}
+
 // The step whose GEMMs follow its row count: the row plan, then a switch node whose bodies are
 // the rest of the step with each branch's GEMMs (the row plan sets the switch on the device, so
 // a step stays one graph launch without a host round trip).
@@ -437,7 +457,7 @@ dcl_status capture_switch(dcl_ctx* c, cudaGraph_t g) {
   prm.conditional.size = STEP_BRANCHES;
   CUDA_TRY(c, cudaGraphAddNode(&node, g, &rows, nullptr, 1, &prm));
   for (int br = 0; br < STEP_BRANCHES && s == DCL_OK; ++br)
-    s = capture_into(c, prm.conditional.phGraph_out[br], nullptr,
+    if (has_branch(c, br)) s = capture_into(c, prm.conditional.phGraph_out[br], nullptr,
                      [&](Enq& q) { enqueue_forward(c, q, br, true, false); });
   return s;
 }
@@ -460,11 +480,12 @@ dcl_status build_exec(dcl_ctx* c, cudaGraphExec_t* exec, bool with_switch, int b
 
 dcl_status build_graph(dcl_ctx* c) {
   destroy_graphs(c);
-  const bool by_rows = !c->few[0].empty() && c->dcfg.kv_cache;
-  const int fixed = c->few[0].empty() ? (int)STEP_PAIR : step_branch(c->B * c->T, c->few_max);
-  if (!c->profiling) return build_exec(c, &c->gexec, by_rows, fixed, nullptr);
+  int first = -1, n = 0;
   for (int br = 0; br < STEP_BRANCHES; ++br)
-    if (by_rows || br == fixed) {
+    if (has_branch(c, br)) first = first < 0 ? br : first, ++n;
+  if (!c->profiling) return build_exec(c, &c->gexec, n > 1, first, nullptr);
+  for (int br = 0; br < STEP_BRANCHES; ++br)
+    if (has_branch(c, br)) {
       const dcl_status s = build_exec(c, &c->prof[br].exec, false, br, &c->prof[br]);
       if (s != DCL_OK) return s;
     }
@@ -516,6 +537,16 @@ int tile_override(const char* name) {
     s += len + (e ? 1 : 0);
   }
   return 0;
+}
+
+// What one of the step's CTA-pair GEMMs takes for `rows` rows, in K blocks of a 256 x 256 tile.
+double pair_cost(const GemmPlan& p, int rows, int pairs) {
+  if (p.cg != 2) return 0;  // (the down projection of a fused MLP: counted with its gate/up)
+  const long m = (rows + 255) / 256, tiles = m * ((p.N + 255) / 256);
+  const double kb = p.K / 64;
+  if (p.fuse) return 10 + kb * (double)((tiles + m * (p.N2 / 256) * p.splits2 + pairs - 1) / pairs);
+  if (p.ds && 2 * (tiles % pairs) <= pairs) return 10 + kb * (double)(tiles / pairs) + (tiles % pairs ? 0.56 * kb : 0);
+  return 10 + kb / p.splits * (double)((tiles * p.splits + pairs - 1) / pairs);
 }
 
 dcl_status build_plans(dcl_ctx* c) {
@@ -623,6 +654,23 @@ dcl_status build_plans(dcl_ctx* c) {
   c->few[0].clear();
   c->few[1].clear();
   const bool planned = t_qkv == kTilePair && t_o == kTilePair && t_gu == kTilePair && t_down == kTilePair;
+  auto qkv_epi = [&](int l, FewEpi* fq) {
+    fq->out = c->qkv;
+    fq->ldo = nqkv;
+    fq->rope = c->rope_cs;
+    fq->rope_cols = (H + G) * hd;
+    fq->head_dim = hd;
+    fq->row_pos = c->rp.row_pos;
+    fq->row_seq = c->rp.row_seq;
+    if (c->kv_fused) {
+      fq->k_col0 = H * hd;
+      fq->kdst = kbuf_of(l);
+      fq->vdst = vbuf_of(l);
+      fq->G = G;
+      fq->T = c->T;
+      fq->Tp = Tp;
+    }
+  };
   c->few_max = few_rows(std::max(std::max(nqkv, d), 2 * m.ffn_dim), c->num_sms);
   if (planned && (cached || R <= c->few_max)) {
     bool ok = true;
@@ -636,21 +684,7 @@ dcl_status build_plans(dcl_ctx* c) {
         base.m_dev = c->rp.counts;
         base.w_early = 1;
         FewEpi fq = base;
-        fq.out = c->qkv;
-        fq.ldo = nqkv;
-        fq.rope = c->rope_cs;
-        fq.rope_cols = (H + G) * hd;
-        fq.head_dim = hd;
-        fq.row_pos = c->rp.row_pos;
-        fq.row_seq = c->rp.row_seq;
-        if (c->kv_fused) {
-          fq.k_col0 = H * hd;
-          fq.kdst = kbuf_of(l);
-          fq.vdst = vbuf_of(l);
-          fq.G = G;
-          fq.T = c->T;
-          fq.Tp = Tp;
-        }
+        qkv_epi(l, &fq);
         FewEpi fh = base, fa = base;
         fh.out = c->h;
         fh.ldo = d;
@@ -667,8 +701,68 @@ dcl_status build_plans(dcl_ctx* c) {
       c->few[1].clear();
     }
   }
+  // the mid-row GEMMs, and which kernels a step of so many rows takes: the few-row ones up to
+  // few_max, above that those of the shorter estimate (in K blocks of a 256 x 256 tile on the
+  // busiest pair; a pair launch's start and end count ten).  Measured, LLaDA-8B shape, 8 layers
+  // (pair -> mid, us a step): 544 rows 1924 -> 1731, 800 rows 2427 -> 2339, 1056 rows 3112 ->
+  // 2988, but 384 rows 1470 -> 1520, 768 rows 2070 -> 2142; Dream-7B shape: 544 rows 2036 ->
+  // 1814, 1056 rows 3108 -> 2787
+  c->mid.clear();
+  if (planned) {
+    c->mid.assign(4 * m.n_layers, MidPlan{});
+    bool ok = true;
+    for (int l = 0; l < m.n_layers && ok; ++l) {
+      const Layer& L = c->layers[l];
+      FewEpi base;
+      base.m_dev = c->rp.counts;
+      FewEpi fq = base, fh = base, fa = base;
+      qkv_epi(l, &fq);
+      fh.out = c->h;
+      fh.ldo = d;
+      fa.out = c->act;
+      fa.ldo = m.ffn_dim;
+      MidPlan* Q = &c->mid[4 * l];
+      ok = mid_plan(&Q[0], c->xn, R, d, L.wqkv, nqkv, EPI_QKV_ROPE, fq, c->num_sms) == cudaSuccess &&
+           mid_plan(&Q[1], c->attn, R, H * hd, L.wo, d, EPI_RESID_F32, fh, c->num_sms) == cudaSuccess &&
+           mid_plan(&Q[2], c->xn, R, d, L.wgu, 2 * m.ffn_dim, EPI_SWIGLU, fa, c->num_sms) == cudaSuccess &&
+           mid_plan(&Q[3], c->act, R, m.ffn_dim, L.wdown, d, EPI_RESID_F32, fh, c->num_sms) == cudaSuccess;
+    }
+    if (!ok) c->mid.clear();
+  }
+  {
+    const int n = (R + 31) / 32 + 1, pairs = c->num_sms / 2;
+    c->row_tab.assign(5 * (size_t)n, 0);
+    for (int i = 0; i < n; ++i) {
+      const int rows = std::min(32 * i, R);
+      int br = STEP_PAIR;
+      if (!c->mid.empty() && rows > 0) {
+        double mid = 0, pair = 0;
+        for (int g = 0; g < 4; ++g) {
+          const MidShape sh = mid_shape(rows, c->mid[g].N, c->mid[g].K, c->mid[g].epi, pairs);
+          c->row_tab[(size_t)(1 + g) * n + i] = (uint16_t)(sh.tt + 256 * sh.splits);
+          mid += sh.cost;
+          pair += pair_cost(c->plans[g], rows, pairs);
+        }
+        if (mid < 0.985 * pair) br = STEP_MID;
+      }
+      if (!c->few[0].empty() && rows <= c->few_max) br = rows <= 32 ? STEP_FEW32 : STEP_FEW;
+      c->row_tab[i] = (uint16_t)br;
+    }
+    if (c->row_tab.size() > c->row_tab_n) {
+      CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+      dev_free_one(c, c->row_tab_dev);
+      c->row_tab_n = 0;
+      c->row_tab_dev = static_cast<uint16_t*>(dev_alloc(c, 2 * c->row_tab.size()));
+      if (!c->row_tab_dev) return fail(c, DCL_ERR_OOM, "row table allocation failed");
+      c->row_tab_n = c->row_tab.size();
+    }
+    CUDA_TRY(c, cudaMemcpyAsync(c->row_tab_dev, c->row_tab.data(), 2 * c->row_tab.size(), cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    for (size_t i = 0; i < c->mid.size(); ++i) c->mid[i].shapes = c->row_tab_dev + (1 + i % 4) * (size_t)n;
+  }
   // split-K counters and partials, shared by the step's GEMMs (they run one after another)
   size_t need_f = 0, need_w = 0;
+  for (const MidPlan& p : c->mid) need_f = std::max(need_f, p.flags_needed);
   for (const GemmPlan& p : c->plans) {
     need_f = p.flags_needed > need_f ? p.flags_needed : need_f;
     need_w = p.ws_needed > need_w ? p.ws_needed : need_w;
@@ -690,6 +784,7 @@ dcl_status build_plans(dcl_ctx* c) {
     if (!c->gemm_ws) return fail(c, DCL_ERR_OOM, "split-K workspace allocation failed");
     c->gemm_ws_n = need_w;
   }
+  for (MidPlan& p : c->mid) p.flags = c->gemm_flags;
   for (GemmPlan& p : c->plans)
     if (gemm_bind_scratch(&p, c->gemm_flags, c->gemm_ws) != cudaSuccess)
       return fail(c, DCL_ERR_CUDA, "GEMM scratch binding failed");

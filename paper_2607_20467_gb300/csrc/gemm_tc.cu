@@ -435,55 +435,6 @@ constexpr int DS_ROW_BYTES = 64 * 4 + 16;
 constexpr int DS_BLOCK_BYTES = 32 * DS_ROW_BYTES;
 static_assert(16 * DS_BLOCK_BYTES <= RING2_BYTES, "the received sum lives in the operand ring");
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int x, int y,
-                                                 uint32_t bar_cluster) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(bar_cluster)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_alloc_pair(uint32_t holder, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(holder), "r"(ncols)
-               : "memory");
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                               uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// arrive (once) on the mbarrier at this offset in every CTA of cta_mask
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint16_t cta_mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          bar),
-      "h"(cta_mask)
-      : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster) : "memory");
-}
 // Bulk copy of `bytes` (a multiple of 16) from this CTA's shared memory to another CTA's
 // (dst and bar: shared::cluster addresses from mapa), completing on that CTA's barrier.
 __device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
@@ -814,26 +765,6 @@ __device__ __forceinline__ void store_partial_pair(const Src& s, Stage& o, const
   o.live = live;
 }
 
-__device__ __forceinline__ void epilogue_bar() {  // the 128 epilogue threads (warps 2..5)
-  asm volatile("bar.sync 1, 128;" ::: "memory");
-}
-// Bounded wait until the counter at f reaches target; false on timeout or abort.
-__device__ __noinline__ bool wait_flag_geq(const int* f, int target, volatile int* abort_flag) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-  if (v >= target) return true;
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    __nanosleep(100);
-    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-    if (v >= target) return true;
-    if ((it & 15u) == 0) {
-      if (*abort_flag) return false;
-      if (globaltimer() - t0 > kWaitLimitNs) return false;
-    }
-  }
-}
-
 // Stream-K fix-up, per epilogue warp.  A tile's last K segment is its CTA pair's last
 // work item, so when it is reached the operand ring is idle in both CTAs and the second
 // TMEM accumulator is free.  Each warp streams the n earlier partials of its 32 rows
@@ -1103,7 +1034,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
-  const uint32_t crank = cluster_ctarank();
+  const uint32_t crank = cluster_rank();
   const uint32_t rank = crank & 1u;             // 0: leader of the pair (issues the MMAs), 1: peer
   const uint32_t lead = crank & ~1u;            // cluster rank of this pair's leader
   const uint16_t pair_mask = (uint16_t)(0x3u << lead);
@@ -1136,7 +1067,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   if (warp == 1) tmem_alloc_pair(holder, TMEM2_COLS);
   tc_fence_before();
   __syncthreads();
-  cluster_sync_all();  // the peer's barriers exist before any remote arrive
+  cluster_sync();  // the peer's barriers exist before any remote arrive
   tc_fence_after();
   const uint32_t tmem_base = *holder_ptr;
   pdl_wait();  // the previous kernel of the step has completed
@@ -1222,7 +1153,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           break;
         }
         if (leader) {
-          const uint32_t full_leader = mapa_shared(full0 + 8 * stage, lead);
+          const uint32_t full_leader = map_cluster(full0 + 8 * stage, lead);
           if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * stage, stage_tx);
 #pragma unroll
           for (int a = 0; a < KA2; ++a) {
@@ -1378,7 +1309,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         const uint32_t partner = crank ^ 2u;
         if (lane == 0) {
           for (int c = 0; c < 2; ++c) mbar_arrive_expect_tx(ds_data0 + 8 * (4 * q + 2 * mine + c), DS_BLOCK_BYTES);
-          mbar_arrive_cluster(mapa_shared(ds_go, partner));
+          mbar_arrive_cluster(map_cluster(ds_go, partner));
         }
         __syncwarp();
         bool go = false;
@@ -1407,8 +1338,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             __syncwarp();
           }
           if (lane == 0 && !*abort_flag) {
-            bulk_copy_to_cluster(mapa_shared(blk, partner), blk, DS_BLOCK_BYTES,
-                                 mapa_shared(ds_data0 + 8 * (4 * q + chunk), partner));
+            bulk_copy_to_cluster(map_cluster(blk, partner), blk, DS_BLOCK_BYTES,
+                                 map_cluster(ds_data0 + 8 * (4 * q + chunk), partner));
             bulk_commit();
           }
         }
@@ -1499,7 +1430,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive_cluster(mapa_shared(tempty0 + 8 * ab, lead));
+      if (lane == 0) mbar_arrive_cluster(map_cluster(tempty0 + 8 * ab, lead));
     }
     if (lane == 0) bulk_wait_read<0>();  // the staging boxes outlive every store reading them
     __syncwarp();
@@ -1508,7 +1439,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
   tc_fence_before();
   __syncthreads();
   __syncwarp();
-  cluster_sync_all();  // no CTA leaves while its pair may still touch its smem or TMEM
+  cluster_sync();  // no CTA leaves while its pair may still touch its smem or TMEM
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem_base, TMEM2_COLS);

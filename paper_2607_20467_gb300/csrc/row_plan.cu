@@ -12,7 +12,8 @@ namespace {
 __global__ void __launch_bounds__(1024) row_plan_kernel(RowPlan rp, const int32_t* __restrict__ p, int B, int N,
                                                         int T, int Bk, int cached, int update,
                                                         int32_t* __restrict__ x, int window, int mask_id,
-                                                        cudaGraphConditionalHandle select, int few_max) {
+                                                        cudaGraphConditionalHandle select,
+                                                        const uint16_t* __restrict__ branches) {
   pdl_wait();
   pdl_launch_dependents();
   extern __shared__ int lm_off[];  // [B], then the sequences' first computed positions [B]
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(1024) row_plan_kernel(RowPlan rp, const int32_
     }
     rp.counts[0] = off;
     rp.counts[1] = lmoff;
-    if (select) cudaGraphSetConditional(select, step_branch(off, few_max));
+    if (select) cudaGraphSetConditional(select, branches[(off + 31) >> 5]);
   }
   __syncthreads();
   for (int b = 0; b < B; ++b) {
@@ -75,11 +76,11 @@ __global__ void __launch_bounds__(1024) row_plan_kernel(RowPlan rp, const int32_
 
 cudaError_t row_plan_launch(const RowPlan& rp, const int32_t* p, int batch, int N, int T, int block_len, int cached,
                             int update, int32_t* x, int window, int mask_id,
-                            cudaGraphConditionalHandle select, int few_max, cudaStream_t stream) {
+                            cudaGraphConditionalHandle select, const uint16_t* branches, cudaStream_t stream) {
   if (batch <= 0 || batch > 4096 || (cached && block_len <= 0) || cached < 0 || cached > 2 || (cached == 2 && !x))
     return cudaErrorInvalidValue;
   return launch_pdl(row_plan_kernel, 1, 1024, 2 * sizeof(int) * batch, stream, rp, p, batch, N, T, block_len, cached,
-                    update, x, window, mask_id, select, few_max);
+                    update, x, window, mask_id, select, branches);
 }
 
 }  // namespace dcl
