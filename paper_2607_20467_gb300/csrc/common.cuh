@@ -159,6 +159,8 @@ cudaError_t gemm_bind_scratch(GemmPlan* plan, int* flags, float* ws);
 // output, the positions / sequences of its rows given by ep.row_pos / ep.row_seq; false
 // (plan unchanged) when the shape does not allow it (T a multiple of 32 is needed).
 bool gemm_fuse_kv(GemmPlan* plan, void* kbuf, void* vt, int batch, int T, int H, int G, int hd, int Tp);
+// Read A from another buffer of `rows` (>= M) rows; the plan's M stays.
+bool gemm_rebind_a(GemmPlan* plan, const void* A, int rows);
 cudaError_t gemm_launch(const GemmPlan& plan, int* err, cudaStream_t stream);
 // Bounded-wait self-test (which = 0: an mbarrier, 1: a global counter; flag = a zero int).
 cudaError_t wait_selftest_launch(int which, const int* flag, int* err, cudaStream_t stream);

@@ -1474,8 +1474,20 @@ dcl_status dcl_op_lmhead_top2(dcl_ctx* c, const void* x_dev, const void* w_dev, 
   const char* why = nullptr;
   if (gemm_plan(&pl, x_dev, R, d, w_dev, V, EPI_LMHEAD, ep, c->num_sms, tile, &why))
     return fail(c, DCL_ERR_INVALID_ARG, "%s", why ? why : "bad LM-head shape");
+  // Up to 16 rows are copied into 32 (the rest zero, never stored): while every CTA streams
+  // weights, boxes of an operand of so few rows arrive late (V = 126464, d = 4096: 1 row 276 us,
+  // 7 rows 218 to 245, from 16 rows on 168; padded 166)
+  const bool pad = R <= 16 && pl.flags_needed == 0 && pl.ws_needed == 0;
+  const size_t x_bytes = pad ? 2 * (size_t)32 * d : 0;
   OpScratch mem(c);
-  if (!mem.get(part_bytes + gemm_scratch_bytes(pl))) return fail(c, DCL_ERR_OOM, "partials allocation failed");
+  if (!mem.get(part_bytes + gemm_scratch_bytes(pl) + x_bytes)) return fail(c, DCL_ERR_OOM, "partials allocation failed");
+  if (pad) {
+    uint8_t* x32 = static_cast<uint8_t*>(mem.ptr) + part_bytes;
+    const size_t live = 2 * (size_t)R * d;
+    CUDA_TRY(c, cudaMemcpyAsync(x32, x_dev, live, cudaMemcpyDeviceToDevice, c->stream));
+    CUDA_TRY(c, cudaMemsetAsync(x32 + live, 0, x_bytes - live, c->stream));
+    if (!gemm_rebind_a(&pl, x32, 32)) return fail(c, DCL_ERR_CUDA, "LM-head operand map failed");
+  }
   float4* part = static_cast<float4*>(mem.ptr);
   float* upart = entropy_dev ? reinterpret_cast<float*>(part + (size_t)R * nblk) : nullptr;
   pl.ep.out = part;

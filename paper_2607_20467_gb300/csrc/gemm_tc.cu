@@ -1627,12 +1627,7 @@ cudaError_t gemm_plan(GemmPlan* plan, const void* A, int M, int K, const void* W
       splits = forced_splits > 0 ? forced_splits : split_auto;
     }
   } else if (bn == 0) {
-    // (the LM head of at most 128 rows is a weight stream whose tiles all take the same time:
-    // whichever form leaves less of its last round empty, V = 126464: 494 tiles on 152 SMs or on
-    // 76 pairs, 175 us against 160)
-    const bool pair_fuller = epi == EPI_LMHEAD && pairs >= 1 &&
-                             wave_efficiency(pair_tiles, pairs) > wave_efficiency(pair_tiles, num_sms);
-    if ((M > BM && pairs >= 1) || pair_fuller) {
+    if (M > BM && pairs >= 1) {
       bn = 256;
       cg = 2;
       splits = split_auto;
@@ -1887,6 +1882,10 @@ cudaError_t gemm_bind_scratch(GemmPlan* p, int* flags, float* ws) {
       return cudaErrorInvalidValue;
   }
   return cudaSuccess;
+}
+
+bool gemm_rebind_a(GemmPlan* p, const void* A, int rows) {
+  return rows >= p->M && !(reinterpret_cast<uintptr_t>(A) & 15) && encode_kmajor(&p->ta, A, rows, p->K, BM);
 }
 
 // Fault-handling self-test: one thread waits, through the same bounded helpers the
