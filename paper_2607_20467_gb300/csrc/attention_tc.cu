@@ -22,9 +22,9 @@
 // its scores and the halves' maxima have been read.  Two tiles per CTA keep four such warps on
 // every scheduler and load each key block once for 256 rows.
 // Measured against one tile per CTA with eight softmax warps (kernel, us): 8 x 1536 positions,
-// 32 heads of 128: 430 -> 289 (1070 TFLOP/s); 4 x 1000, 28 q / 4 kv heads: 81 -> 55; 1 x 512: 9.3
+// 32 heads of 128: 430 -> 281 (1100 TFLOP/s); 4 x 1000, 28 q / 4 kv heads: 81 -> 55; 1 x 512: 9.3
 // -> 9.7; 32 query rows of each of 16 x 896 (28 / 4 heads): 55 -> 14; 32 rows of 1 x 1536: 18.9
-// -> 10.4.
+// -> 10.1.
 //
 // Where the units of a launch leave SMs idle the key axis is split over the S CTAs of a
 // cluster: each keeps (m, l, O) of its blocks, and after one cluster barrier every CTA
@@ -35,9 +35,9 @@
 //
 // Roles (576 threads): warp 0 lane 0 TMA producer (Q once, then K / V^T blocks through a ring
 // in the order the MMAs consume them); warp 1 allocates TMEM and issues the MMAs (a second
-// issuer, a warp per tile, gained nothing); warps 2..17 run the softmax and the epilogue (TMEM lane quarter = band of the tile).  V enters
-// as V^T (a K-major operand, kv contiguous, fp16), written by the QKV GEMM's epilogue or by
-// v_transpose_kernel from the q|k|v buffer.
+// issuer, a warp per tile, gained nothing); warps 2..17 run the softmax and the epilogue (TMEM
+// lane quarter = band of the tile).  V enters as V^T (a K-major operand, kv contiguous, fp16),
+// written by the QKV GEMM's epilogue or by v_transpose_kernel from the q|k|v buffer.
 // Every wait is bounded (DERR_WAIT_TIMEOUT).
 #include <algorithm>
 
@@ -144,10 +144,54 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int S = (int)cluster_size(), rank = (int)cluster_rank();
-  // grid (rank, kv head, unit-major sequence): the unit is the slowest index, so that the CTAs
-  // with work come first in dispatch order
-  const int g = blockIdx.y, b = blockIdx.z % B, zc = blockIdx.z / B;
+  // grid ((unit, sequence, kv head) x rank, one dimension): the unit is the slowest index, so
+  // that the CTAs with work come first in dispatch order
+  const int cl = (int)blockIdx.x / S, g = cl % G, b = cl / G % B, zc = cl / G / B;
   const int rep = H / G, nb = (T + 127) / 128;
+
+  int q_off, q_len, nch, nbands, band0;
+  bool split;
+  // This CTA's rows, once the previous kernels of the step (the row plan among them) have
+  // completed; false if it has none (then the whole cluster, if split): uniform over the CTA.
+  auto plan = [&]() {
+    pdl_wait();
+    pdl_launch_dependents();
+    // the query rows of sequence b are rows [off, off + len) of q and of the output
+    // (without tables its last q_rows positions)
+    q_off = seq_off ? seq_off[b] : b * T + T - q_rows;
+    q_len = seq_len ? seq_len[b] : q_rows;
+    split = mode == ATTN_SPLIT;
+    if (mode == ATTN_BY_ROWS) {
+      // the cheapest of whole or split units of eight or four bands that the grid has CTAs for
+      int total[2] = {0, 0}, most[2] = {0, 0};  // of eight, of four
+      for (int i = lane; i < B; i += 32)
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int n = attn_units(seq_len[i], rep, 8 >> k);
+          total[k] += n;
+          most[k] = max(most[k], n);
+        }
+      const int Z = (int)gridDim.x / S / G / B;
+      long best = 0;
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int n = (int)__reduce_add_sync(0xffffffffu, (unsigned)total[k]) * G;
+        const int mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)most[k]);
+        const long whole = attn_cost(n, 8 >> k, nb, 1), parts = attn_cost(n, 8 >> k, nb, S);
+        if (k == 0 || (mx <= Z * S && whole < best)) best = whole, bands = 8 >> k, split = false;
+        if (mx <= Z && S > 1 && parts < best) best = parts, bands = 8 >> k, split = true;
+      }
+    }
+    nch = (q_len + 31) / 32;  // band i: head i / nch, rows 32 (i % nch) ..
+    nbands = rep * nch;
+    band0 = (split ? zc : zc * S + rank) * bands;
+    return band0 < nbands;
+  };
+  // Where the rows are the row plan's, CTAs past each sequence's first cluster may well have
+  // none: those look first and leave without a set-up (with it the empty CTAs of a T = 512 step
+  // outlasted the others: 12.6 against 9.5 us).
+  const bool look_first = mode == ATTN_BY_ROWS && zc > 0;
+  if (look_first && !plan()) return;
 
   // set-up first (it reads nothing that earlier kernels write), so that under programmatic
   // dependent launch it overlaps the tail of the kernel before
@@ -177,37 +221,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *holder_ptr;
 
-  pdl_wait();  // the previous kernels of the step (the row plan among them) have completed
-  pdl_launch_dependents();
-  // the query rows of sequence b are rows [off, off + len) of q and of the output
-  // (without tables its last q_rows positions)
-  const int q_off = seq_off ? seq_off[b] : b * T + T - q_rows;
-  const int q_len = seq_len ? seq_len[b] : q_rows;
-  bool split = mode == ATTN_SPLIT;
-  if (mode == ATTN_BY_ROWS) {
-    // the cheapest of whole or split units of eight or four bands that the grid has CTAs for
-    int total[2] = {0, 0}, most[2] = {0, 0};  // of eight, of four
-    for (int i = lane; i < B; i += 32)
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int n = attn_units(seq_len[i], rep, 8 >> k);
-        total[k] += n;
-        most[k] = max(most[k], n);
-      }
-    const int Z = gridDim.z / B;
-    long best = 0;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int n = (int)__reduce_add_sync(0xffffffffu, (unsigned)total[k]) * G;
-      const int mx = (int)__reduce_max_sync(0xffffffffu, (unsigned)most[k]);
-      const long whole = attn_cost(n, 8 >> k, nb, 1), parts = attn_cost(n, 8 >> k, nb, S);
-      if (k == 0 || (mx <= Z * S && whole < best)) best = whole, bands = 8 >> k, split = false;
-      if (mx <= Z && S > 1 && parts < best) best = parts, bands = 8 >> k, split = true;
-    }
-  }
-  const int nch = (q_len + 31) / 32, nbands = rep * nch;  // band i: head i / nch, rows 32 (i % nch) ..
-  const int band0 = (split ? zc : zc * S + rank) * bands;
-  if (band0 >= nbands) {  // nothing to do (all CTAs of the cluster, if split): uniform over the CTA
+  if (!look_first && !plan()) {
     if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
     return;
   }
@@ -620,7 +634,9 @@ cudaError_t launch_attn(const AttnPlan& p, const AttnRows& rows, int* err, cudaS
   }
   const AttnShape a = attn_shape(p, rows);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.S, p.G, a.Z * p.batch);
+  const long grid = (long)a.S * p.G * a.Z * p.batch;
+  if (grid > 0x7fffffffl) return cudaErrorInvalidValue;
+  cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(AT_THREADS);
   cfg.dynamicSmemBytes = AttnCfg<HD>::SMEM;
   cfg.stream = stream;

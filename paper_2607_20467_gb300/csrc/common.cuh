@@ -248,7 +248,7 @@ struct AttnPlan {
   int batch = 0, T = 0, H = 0, G = 0, hd = 0, kcol0 = 0;
 };
 // What a launch knows of its query rows: at most `most` of a sequence (exact: each has that
-// many) and `total` of all; seqs: the sequences that have any, as far as the launch is laid out
+// many, or with tables none) and `total` of all; seqs: the sequences that have any, as far as the launch is laid out
 // for (more are taken, less evenly).
 struct AttnRows {
   int most = 0, total = 0, seqs = 1;

@@ -298,7 +298,7 @@ void enqueue_forward(dcl_ctx* c, Enq& q, int branch, bool with_dcv, bool snapsho
   ar.most = std::min(c->T, rows);
   ar.total = rows;
   ar.seqs = c->kv_fused ? std::min(c->B, std::max(1, rows / 32)) : c->B;
-  ar.exact = !c->kv_fused;
+  ar.exact = !c->dcfg.kv_cache;  // (a finished sequence then has none: its units leave at once)
   if (h_in) {
     if (q.err == cudaSuccess)
       q.err = cudaMemcpyAsync(c->h, h_in, sizeof(float) * R * d, cudaMemcpyDeviceToDevice, c->stream);

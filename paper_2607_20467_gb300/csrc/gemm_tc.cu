@@ -9,7 +9,7 @@
 //                   BNx64 W box (128-byte swizzle) land in a STAGES-deep smem ring,
 //                   completing a transaction-count mbarrier.
 //   warp 1        : allocates TMEM (2 x BN fp32 columns: double-buffered accumulator);
-//                   lane 0 issues tcgen05.mma (M=128, N=BN, K=16) x4 per K block and
+//                   one lane issues tcgen05.mma (M=128, N=BN, K=16) x4 per K block and
 //                   tcgen05.commit to release smem stages / publish finished tiles.
 //   warps 2..5    : epilogue.  Warp w reads TMEM lanes 32*(w%4)..+31 (one output row
 //                   per thread) with tcgen05.ld and applies the fused epilogue while the
@@ -1677,10 +1677,9 @@ cudaError_t gemm_plan(GemmPlan* plan, const void* A, int M, int K, const void* W
   // Half-width tail (on request, kTileHalves): whole tiles in full rounds, then each
   // tile of a partial last round as two 256 x 128 pieces on two pairs, with no partial
   // sums to combine (each output is still one MMA chain over all of K, so results are
-  // bit-identical to whole tiles).  Measured, a piece takes as long per K block as a
-  // whole tile: the six-stage operand ring, not the tensor core, sets the pace of a
-  // K block (about 1.7 us of load latency under full load over six 32 KB stages), so the
-  // planner does not pick it.
+  // bit-identical to whole tiles).  Measured (while a diverged thread issued the loads and
+  // the MMAs, about 550 cycles a K block whatever its width), a piece took as long per K
+  // block as a whole tile; the planner does not pick it.
   int halves = 0;
   if (cg == 2 && pair_forced && (tile & kTileHalves)) {
     if (streamk != 0 || epi == EPI_LMHEAD || forced_splits > 1) {

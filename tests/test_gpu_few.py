@@ -109,3 +109,29 @@ def test_step_matches_the_pair_gemms(ctx, monkeypatch, hd, N, M, B, cache, offse
         a, b = a.double(), b.double()
         rel = (a - b).norm(dim=1) / b.norm(dim=1)
         assert rel.max() <= 2 * 2 * 3.5e-3, rel.max()
+
+
+def test_a_finished_sequence_leaves_its_neighbour_alone(ctx):
+    """Sequences of 127 positions: with the first finished the step
+    computes the second's rows only, from other places of every buffer, to the same bits."""
+    import paper_2607_20467_gb300 as dcl
+    import synthetic as syn
+    m = MODELS[64]
+    shape = syn.ModelShape(2, m["d"], m["H"], m["G"], 64, m["F"], 4096, 4095, 1e4)
+    N, M, B = 37, 90, 2
+    x, p = syn.decode_state(3, syn.prompt_ids(3, B, N, 4095), M, 21, M // 2, 4095)
+    with dcl.Context(shape, max_batch=B, max_seq=N + M) as c:
+        c.init_random_weights(7, 0.02, 2.0, 0.1)
+        c.set_prompt(x[:, :N], dcl.decode_config(tau_commit=1.0, tau_draft=1.0, min_commit=0, gen_len=M))
+        both, other, alone = (torch.zeros(B, M, device="cuda") for _ in range(3))
+        c.set_state(x, p)
+        c.forward_debug(p1=both)
+        y = x.copy()
+        y[1, N:N + 20] = 11
+        c.set_state(y, p)
+        c.forward_debug(p1=other)  # other contents everywhere
+        x[0, N:], p[0] = 5, N + M
+        c.set_state(x, p)
+        c.forward_debug(p1=alone)
+        assert torch.equal(both[1], alone[1])
+        assert not torch.equal(both[1], other[1])
