@@ -742,7 +742,7 @@ def run_ours(args):
         "clocks": clocks,
         "e2e": {"value": world * B * M / e2e_mean, "unit": "tokens/s",
                 "h2d_bytes_per_step": 4 * B * T + 12 * B + 4,
-                "d2h_bytes_per_step": 4 * B * M + 8 * B + 4 * (statistics.mean(e2e_steps) + 1),
+                "d2h_bytes_per_step": 4 * B * M + 12 * B + 8,
                 "step": "one dcl_set_prompt + dcl_generate call (a whole generation)",
                 "ms_per_generation": 1e3 * e2e_mean, "steps_per_generation": statistics.mean(e2e_steps)},
         "cpu_baseline": cpu,
