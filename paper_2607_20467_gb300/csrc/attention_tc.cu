@@ -11,7 +11,9 @@
 // in fp32, P written to shared memory in fp16 (11 significant bits; P <= 2^8), and O += P V in
 // TMEM with V^T held in fp16 (the bf16 values of v, which fp16 holds exactly).  m moves only
 // when a block's maximum exceeds it by more than 8 (P stays below 2^8); l and O are then scaled
-// by the same factor, so O / l is unchanged.  O / l leaves through TMA.
+// by the same factor, so O / l is unchanged.  m is held and exchanged in fp32: P passes 2^8 by as
+// much as m misses the maximum (an m rounded to bf16 gave infinities from scores of about 1400
+// on).  O / l leaves through TMA.
 //
 // What bounds it now is shared memory: per key block of two tiles the products read 256 KB of
 // operands, P is written (64 KB) and the block arrives (64 KB), 3072 cycles at 128 bytes a cycle
@@ -62,8 +64,10 @@ struct AttnCfg {
   static constexpr int P_BYTES = 2 * AT_BOX;        // a tile of P (fp16) [128][128]
   static constexpr int BARS = 256;
   static constexpr int DATA = 2 * Q_BYTES + STAGES * STAGE_BYTES + 2 * P_BYTES;
-  static constexpr int RED = 2 * 2 * 128 * 2;       // row maxima of the halves [tile][half][row], bf16
-  static constexpr size_t SMEM = 1024 + (size_t)DATA + BARS + RED;
+  static constexpr int RED = 2 * 2 * 128 * 4;       // row maxima of the halves [tile][half][row]
+  // (no slack for the 1024-byte alignment, which the declaration asks for and the kernel checks:
+  // 2 x 1 KB of fp32 maxima do not fit beside it)
+  static constexpr size_t SMEM = (size_t)DATA + BARS + RED;
   static constexpr uint32_t TMEM_COLS = 512;        // S of two tiles (2 x 128), O of two (2 x HD)
   // a split's parts: O rows in fp32 (padded by 16 bytes), then {m, l} of every row
   static constexpr int O_PITCH = HD * 4 + 16;
@@ -121,14 +125,20 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
                    const int* __restrict__ seq_off, const int* __restrict__ seq_len, int q_rows, int mode, int bands,
                    int* err) {
   using C = AttnCfg<HD>;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  uint8_t* smem = smem_raw + (base - raw);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  // (opaque to the compiler: with a known constant in every address it spills, 3 % of the time)
+  uint32_t base = smem_u32(smem_raw);
+  asm volatile("" : "+r"(base));
+  uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
+  if (base & 1023u) {  // (the swizzled operands need it; uniform over the grid)
+    if (threadIdx.x == 0) report_error(err, DERR_BAD_SHAPE);
+    return;
+  }
   const uint32_t sQ = base;                                // per tile: KB boxes
   const uint32_t sKV = sQ + 2 * C::Q_BYTES;
   const uint32_t sP = sKV + C::STAGES * C::STAGE_BYTES;    // per tile: two 64-key boxes of P
-  const uint32_t bars = base + C::DATA;
+  const uint32_t red = base + C::DATA;                     // the halves' row maxima
+  const uint32_t bars = red + C::RED;
   const uint32_t q_full = bars;
   const uint32_t kv_full0 = bars + 8;                      // + 8 s
   const uint32_t kv_empty0 = kv_full0 + 8 * C::STAGES;     // + 8 s
@@ -140,7 +150,6 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
   const uint32_t holder = drain + 8;
   volatile uint32_t* holder_ptr = reinterpret_cast<volatile uint32_t*>(smem + (holder - base));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + (holder + 4 - base));
-  __nv_bfloat16* red = reinterpret_cast<__nv_bfloat16*>(smem + C::DATA + C::BARS);
 
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int S = (int)cluster_size(), rank = (int)cluster_rank();
@@ -366,8 +375,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
     const uint32_t sPt = sP + tile * C::P_BYTES;
     const uint32_t s_full = s_full0 + 8 * tile, s_empty = s_empty0 + 8 * tile, p_full = p_full0 + 8 * tile,
                    p_empty = p_empty0 + 8 * tile;
-    __nv_bfloat16* mine = red + (tile * 2 + hs) * 128 + r;
-    const __nv_bfloat16* other = red + (tile * 2 + (hs ^ 1)) * 128 + r;
+    const uint32_t top = red + (uint32_t)(4 * ((tile * 2 + hs) * 128 + r));  // (the other half's: ^ 512)
     auto band_bar = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1u + 4u * tile + q) : "memory"); };  // the band's two warps
     constexpr int OH = HD / 2;  // O columns of this warp: [hs * OH, + OH)
     const float scale2 = kLog2e * rsqrtf((float)HD);
@@ -407,12 +415,10 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
           }
           mm = max3f(mx[0], mx[1], fmaxf(mx[2], mx[3])) * scale2;
         }
-        // the halves agree on a maximum; its bf16 rounding serves (any m that both use will do,
-        // and P stays below 2^9)
-        const __nv_bfloat16 own = __float2bfloat16_rn(mm);
-        *mine = own;
+        // the halves agree on the block's maximum
+        st_shared_f32(top, mm);
         band_bar();
-        const float mb = fmaxf(__bfloat162float(own), __bfloat162float(*other));
+        const float mb = fmaxf(mm, ld_shared_f32(top ^ 512u));
         __syncwarp();
         if (lane == 0 && ok) mbar_arrive(s_empty);  // scores and maxima read: the next block's may be written
         if (ok) {

@@ -62,3 +62,20 @@ def test_late_maximum(ops, qr):
     x[:, :H, 0] = 8.0
     x[:, H:H + G, 0] = (torch.arange(T, device="cuda") / 16)[:, None]  # adds up to 48 to a score
     _check(ops, x.view(B * T, -1).to(torch.bfloat16).contiguous(), B, T, H, G, hd, qr)
+
+
+@pytest.mark.parametrize("base", [-2.0 ** 14, -2.0 ** 10, 2.0 ** 10, 2.0 ** 14])
+@pytest.mark.parametrize("B,T,H,G,hd,qr", [(8, 300, 16, 16, 128, 0), (8, 300, 16, 16, 64, 0),  # whole
+                                           (1, 1100, 4, 2, 128, 32), (1, 1100, 4, 2, 64, 32)])  # split
+def test_large_scores(ops, B, T, H, G, hd, qr, base):
+    """Scores near +-10^3 and +-10^4 that differ by a few within a block, and along the keys by up
+    to 12 in 16 steps: the reference maximum has to follow them exactly, P being held in fp16.
+    q and k are small integers and powers of two, so q k^T is exact in fp32 (integers below 2^18)
+    and the tolerance that of small scores."""
+    g = torch.Generator(device="cuda").manual_seed(11)
+    q, k = (torch.randint(-2, 3, (B * T, n, hd), generator=g, device="cuda").float() for n in (H, G))
+    root = 8.0  # q k^T / root: base + steps (sqrt(hd) for hd = 64; for 128 the scores are 0.71 of that)
+    q[..., 0], k[..., 0] = base / 128, 128.0 * root           # every score: base
+    q[..., 1], k[..., 1] = 1.0, 6.0 * ((torch.arange(B * T, device="cuda") * 16 // T) % 16)[:, None]
+    v = torch.randn(B * T, G, hd, generator=g, device="cuda")
+    _check(ops, torch.cat([q, k, v], 1).view(B * T, -1).to(torch.bfloat16).contiguous(), B, T, H, G, hd, qr)
