@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(MD_THREADS, 1)
     MidItem it;
     for (int idx = 0; item(idx, it); ++idx) {
       const int ab = idx & 1;
-      if (!mbar_wait(tfull0 + 8 * ab, (uint32_t)(idx >> 1) & 1u, abort_flag)) {
+      if (!epilogue_wait(tfull0 + 8 * ab, (uint32_t)(idx >> 1) & 1u, abort_flag)) {
         *abort_flag = 1;
         report_error(err, DERR_WAIT_TIMEOUT);
         break;

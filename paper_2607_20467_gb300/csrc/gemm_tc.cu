@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
       const int ab = j & 1;
       const uint32_t aph = (uint32_t)(j >> 1) & 1u;
-      if (!mbar_wait(tfull0 + 8 * ab, aph, abort_flag)) {
+      if (!__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * ab, aph, abort_flag))) {
         *abort_flag = 1;
         report_error(err, DERR_WAIT_TIMEOUT);
         break;
@@ -1249,7 +1249,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     for (int idx = 0; next_item(idx, sc, cluster, it); ++idx) {
       const int ab = idx & 1;
       const uint32_t aph = (uint32_t)(idx >> 1) & 1u;
-      if (!mbar_wait(tfull0 + 8 * ab, aph, abort_flag)) {
+      if (!epilogue_wait(tfull0 + 8 * ab, aph, abort_flag)) {
         *abort_flag = 1;
         report_error(err, DERR_WAIT_TIMEOUT);
         break;
