@@ -1438,6 +1438,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  if (*abort_flag) abort_grace();
   __syncwarp();
   cluster_sync();  // no CTA leaves while its pair may still touch its smem or TMEM
   if (warp == 1) {

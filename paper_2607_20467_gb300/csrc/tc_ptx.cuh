@@ -376,6 +376,14 @@ __device__ __noinline__ bool epilogue_wait(uint32_t bar, uint32_t parity, volati
       : "+r"(ok)::"memory");
   return ok != 0;
 }
+// On the way out of an aborted CTA of a pair: the copies in flight to its shared memory land
+// (microseconds) before that goes to another block.  By time, as they complete on a barrier of
+// the pair's leader, which an abort may leave without its own arrival, so that it never flips.
+constexpr uint64_t kAbortGraceNs = 10000000ull;  // 10 ms
+__device__ __noinline__ void abort_grace() {
+  const uint64_t t0 = globaltimer();
+  while (globaltimer() - t0 < kAbortGraceNs) __nanosleep(1000);
+}
 // Bounded wait until the counter at f reaches target; false on timeout or abort.
 __device__ __noinline__ bool wait_flag_geq(const int* f, int target, volatile int* abort_flag) {
   int v;
