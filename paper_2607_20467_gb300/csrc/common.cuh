@@ -245,7 +245,7 @@ struct AttnPlan {
   __half* vt = nullptr;
   const int* seq_off = nullptr;
   const int* seq_len = nullptr;
-  int batch = 0, T = 0, H = 0, G = 0, hd = 0, kcol0 = 0;
+  int batch = 0, T = 0, H = 0, G = 0, hd = 0, kcol0 = 0, sms = 0;
 };
 // What a launch knows of its query rows: at most `most` of a sequence (exact: each has that
 // many, or with tables none) and `total` of all; seqs: the sequences that have any, as far as the launch is laid out
@@ -258,7 +258,7 @@ enum AttnMode : int { ATTN_WHOLE = 0, ATTN_SPLIT = 1, ATTN_BY_ROWS = 2 };
 int attn_vt_pitch(int T);
 cudaError_t attention_plan(AttnPlan* p, const __nv_bfloat16* qkv, const __nv_bfloat16* kbuf, __half* vt,
                            __nv_bfloat16* out, int batch, int T, int H, int G, int hd, int rows_max,
-                           const int* seq_off, const int* seq_len);
+                           const int* seq_off, const int* seq_len, int num_sms);
 cudaError_t attention_launch(const AttnPlan& p, const AttnRows& rows, int* err, cudaStream_t stream);  // both kernels
 cudaError_t attention_transpose_launch(const AttnPlan& p, cudaStream_t stream);  // v -> vt
 cudaError_t attention_core_launch(const AttnPlan& p, const AttnRows& rows, int* err, cudaStream_t stream);  // attention

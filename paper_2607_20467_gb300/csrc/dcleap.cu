@@ -636,8 +636,8 @@ dcl_status build_plans(dcl_ctx* c) {
   for (int l = 0; l < m.n_layers; ++l) {
     // (without the fused key store the rows are the identity layout b*T + t: no tables)
     if (attention_plan(&c->attn_plans[l], c->qkv, c->kv_fused ? kbuf_of(l) : nullptr, vbuf_of(l), c->attn, c->B, c->T,
-                       H, G, hd, R, c->kv_fused ? c->rp.seq_off : nullptr, c->kv_fused ? c->rp.seq_len : nullptr) !=
-        cudaSuccess)
+                       H, G, hd, R, c->kv_fused ? c->rp.seq_off : nullptr, c->kv_fused ? c->rp.seq_len : nullptr,
+                       c->num_sms) != cudaSuccess)
       return fail(c, DCL_ERR_UNSUPPORTED, "attention plan failed");
   }
   EpiParams el;
@@ -1447,8 +1447,8 @@ dcl_status dcl_op_attention(dcl_ctx* c, const void* qkv_dev, void* out_dev, int3
     return fail(c, DCL_ERR_OOM, "attention scratch allocation failed");
   AttnPlan pl;
   if (attention_plan(&pl, static_cast<const __nv_bfloat16*>(qkv_dev), nullptr, static_cast<__half*>(mem.ptr),
-                     static_cast<__nv_bfloat16*>(out_dev), batch, T, H, G, hd, batch * T, nullptr, nullptr) !=
-      cudaSuccess)
+                     static_cast<__nv_bfloat16*>(out_dev), batch, T, H, G, hd, batch * T, nullptr, nullptr,
+                     c->num_sms) != cudaSuccess)
     return fail(c, DCL_ERR_INVALID_ARG, "attention: operands must be 16-byte aligned");
   AttnRows ar;  // sequence b's queries: positions [T - q_rows, T)
   ar.most = q_rows ? q_rows : T;
