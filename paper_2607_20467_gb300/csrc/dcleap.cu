@@ -1474,10 +1474,13 @@ dcl_status dcl_op_lmhead_top2(dcl_ctx* c, const void* x_dev, const void* w_dev, 
   const char* why = nullptr;
   if (gemm_plan(&pl, x_dev, R, d, w_dev, V, EPI_LMHEAD, ep, c->num_sms, tile, &why))
     return fail(c, DCL_ERR_INVALID_ARG, "%s", why ? why : "bad LM-head shape");
-  // Up to 16 rows are copied into 32 (the rest zero, never stored): while every CTA streams
-  // weights, boxes of an operand of so few rows arrive late (V = 126464, d = 4096: 1 row 276 us,
-  // 7 rows 218 to 245, from 16 rows on 168; padded 166)
-  const bool pad = R <= 16 && pl.flags_needed == 0 && pl.ws_needed == 0;
+  // Up to 16 rows of a large head are copied into 32 (the rest zero, never stored): while every CTA
+  // streams weights, boxes of an operand of so few rows arrive late.  The copy and the zeros take
+  // 4 to 5 us, so only where the column tiles fill most of the GPU and K is long.  A call, us, as it
+  // is -> padded: V = 126464, d = 4096 228 (1 row), 205 (7) -> 196; 32000 x 4096 80 -> 73; 64000 x 2048
+  // 80 -> 73; 32000 x 2048 56 -> 53; but 16000 x 4096 56 -> 61, 126464 x 1536 107 -> 107, 126464 x 768
+  // 68 -> 72, 4097 x 256 31 -> 36
+  const bool pad = R <= 16 && 4L * nblk >= 3L * c->num_sms && d >= 2048 && pl.flags_needed == 0 && pl.ws_needed == 0;
   const size_t x_bytes = pad ? 2 * (size_t)32 * d : 0;
   OpScratch mem(c);
   if (!mem.get(part_bytes + gemm_scratch_bytes(pl) + x_bytes)) return fail(c, DCL_ERR_OOM, "partials allocation failed");
