@@ -140,7 +140,11 @@ typedef struct dcl_ctx dcl_ctx;
  *              step is captured into a CUDA graph on this stream, so it must not be the
  *              legacy default stream itself.
  *   alloc      optional allocator; NULL uses cudaMalloc/cudaFree.
- * Weights are allocated (uninitialised) here: 2 bytes per parameter.
+ * Weights are allocated (uninitialised) here: 2 bytes per parameter.  Scratch of the
+ * single-kernel calls (dcl_op_linear, dcl_op_attention, dcl_op_lmhead_top2, the logits of
+ * dcl_forward_debug) of up to 256 MB stays with the context from call to call, until
+ * dcl_destroy or until another allocation of the context fails (it is then released and the
+ * allocation tried again); larger scratch is allocated and released by the call.
  * Errors: INVALID_ARG, UNSUPPORTED (shape), OOM, CUDA.  *out is NULL on failure. */
 dcl_status dcl_create(const dcl_model_config* cfg, int32_t max_batch, int32_t max_seq,
                       void* cuda_stream, const dcl_allocator* alloc, dcl_ctx** out);

@@ -151,14 +151,27 @@ dcl_status fail(dcl_ctx* c, dcl_status s, const char* fmt, ...) {
       return fail((ctx), DCL_ERR_CUDA, "%s failed: %s", #expr, cudaGetErrorString(e_));     \
   } while (0)
 
+void dev_free_one(dcl_ctx* c, void* ptr);
+
 void* dev_alloc(dcl_ctx* c, size_t bytes) {
-  void* ptr = nullptr;
   if (bytes == 0) bytes = 16;
-  if (c->custom_alloc) {
-    ptr = c->alloc.alloc(bytes, c->alloc.user);
-  } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    ptr = nullptr;
+  auto get = [&]() {
+    void* ptr = nullptr;
+    if (c->custom_alloc) {
+      ptr = c->alloc.alloc(bytes, c->alloc.user);
+    } else if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      ptr = nullptr;
+    }
+    return ptr;
+  };
+  void* ptr = get();
+  if (!ptr && c->op_buf) {  // the kept scratch gives way (no call allocates while it uses it)
+    cudaStreamSynchronize(c->stream);
+    dev_free_one(c, c->op_buf);
+    c->op_buf = nullptr;
+    c->op_cap = 0;
+    ptr = get();
   }
   if (ptr) c->owned.push_back(ptr);
   return ptr;
@@ -231,6 +244,7 @@ struct OpScratch {
       if (c->op_buf) {
         cudaStreamSynchronize(c->stream);  // no launch may still use the old buffer
         dev_free_one(c, c->op_buf);
+        c->op_buf = nullptr;
       }
       c->op_buf = dev_alloc(c, bytes);
       c->op_cap = c->op_buf ? bytes : 0;
