@@ -221,8 +221,7 @@ struct MidPlan {
   int M = 0, N = 0, K = 0, epi = EPI_RESID_F32;
   FewEpi ep;
   int grid = 0;
-  int shape = 0;                     // of M rows: tt + 256 * splits
-  const uint16_t* shapes = nullptr;  // device, by rows / 32 (with ep.m_dev)
+  const uint16_t* shapes = nullptr;  // device, by rows / 32 rounded up: MidShape's tt + 256 * splits
   size_t flags_needed = 0;           // ints of zero-initialised counters
   int* flags = nullptr;
 };

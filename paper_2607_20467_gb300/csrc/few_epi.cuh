@@ -12,9 +12,7 @@ constexpr int FW_TILE = 128;           // weight rows of a CTA's tile
 constexpr int FW_PITCH = FW_TILE + 4;  // fp32 per token of a staged sum
 
 struct FewArgs {
-  int nkb;     // K blocks
-  int nt_max;  // tokens of a token tile at most (32 or FEW_TILE_ROWS)
-  int units, tiles;
+  int nkb;  // K blocks
   int N, M;
   FewEpi ep;
 };

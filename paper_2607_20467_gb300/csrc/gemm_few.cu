@@ -54,10 +54,15 @@ constexpr int FW_RING = (int)FW_SMEM - 1024 - FW_BARS;
 static_assert(FEW_TILE_ROWS * FW_PITCH * 4 <= FW_RING, "the staged sum lives in the operand ring");
 static_assert(8 * (2 * FW_MAX_STAGES + 1) + 16 <= 256, "barrier area");
 
+struct FewTiles {
+  int nt_max;        // tokens of a token tile at most (32 or FEW_TILE_ROWS)
+  int units, tiles;  // tiles of weight rows, of tokens
+};
+
 template <int EPI>
 __global__ void __launch_bounds__(FW_THREADS, 2)
     few_gemm_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tx,
-                    const __grid_constant__ FewArgs a, int* err) {
+                    const __grid_constant__ FewArgs a, const FewTiles cut, int* err) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -72,11 +77,11 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;  // (warp-uniform)
   const int S = (int)cluster_size(), rank = (int)cluster_rank();
   // the cluster's tile of weight rows and its tile of tokens (rows [tok0, tok0 + nt_max))
-  const int u = (int)blockIdx.x / S % a.units, tok0 = (int)blockIdx.x / S / a.units * a.nt_max;
+  const int u = (int)blockIdx.x / S % cut.units, tok0 = (int)blockIdx.x / S / cut.units * cut.nt_max;
   const int kb0 = rank * a.nkb / S, nkb = (rank + 1) * a.nkb / S - kb0;
   // a stage: the weight rows of one K block, then the tokens'.  The stage pitch is that of
   // the most tokens the launch may hold, known before the row count is.
-  const int stage_bytes = FW_W_BYTES + a.nt_max * 128;
+  const int stage_bytes = FW_W_BYTES + cut.nt_max * 128;
   const int stages = min(FW_RING / stage_bytes, FW_MAX_STAGES);
 
   if (threadIdx.x == 0) {
@@ -117,9 +122,9 @@ __global__ void __launch_bounds__(FW_THREADS, 2)
   pdl_wait();
   pdl_launch_dependents();
   const int all = a.ep.m_dev ? min(a.M, *a.ep.m_dev) : a.M;
-  const int rows = max(min(all - tok0, a.nt_max), 0);
+  const int rows = max(min(all - tok0, cut.nt_max), 0);
   int nt = (rows + 31) & ~31;         // the MMA's N
-  if (all > a.tiles * a.nt_max) {     // (the launch is not chosen for so many rows)
+  if (all > cut.tiles * cut.nt_max) {     // (the launch is not chosen for so many rows)
     if (threadIdx.x == 0) report_error(err, DERR_BAD_SHAPE);
     nt = 0;
   }
@@ -264,9 +269,6 @@ cudaError_t launch_few(const FewPlan& p, int* err, cudaStream_t stream) {
   }
   FewArgs a;
   a.nkb = p.K / FW_BK;
-  a.nt_max = p.nt_max;
-  a.units = p.units;
-  a.tiles = p.tiles;
   a.N = p.N;
   a.M = p.M;
   a.ep = p.ep;
@@ -284,7 +286,7 @@ cudaError_t launch_few(const FewPlan& p, int* err, cudaStream_t stream) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kern, p.tw, p.tx, a, err);
+  return cudaLaunchKernelEx(&cfg, kern, p.tw, p.tx, a, FewTiles{p.nt_max, p.units, p.tiles}, err);
 }
 
 }  // namespace

@@ -40,8 +40,7 @@ static_assert(8 * (2 * MD_STAGES + 5) + 8 <= 256, "barrier area");
 
 struct MidArgs {
   FewArgs f;
-  const uint16_t* shapes;  // by rows / 32 (NULL: `shape`)
-  int shape;               // tt + 256 * splits
+  const uint16_t* shapes;  // by rows / 32 rounded up: tt + 256 * splits
   int pair_units;          // tiles of 256 weight rows
   int* flags;              // [tiles][2] ordered-add counters, zero between launches (splits > 1)
 };
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(MD_THREADS, 1)
   pdl_launch_dependents();
 
   const int rows = a.f.ep.m_dev ? min(a.f.M, *a.f.ep.m_dev) : a.f.M;
-  const int shape = a.shapes ? a.shapes[(rows + 31) >> 5] : a.shape;
+  const int shape = a.shapes[(rows + 31) >> 5];
   const int tt = shape & 255, S = shape >> 8;
   const int per = tt ? (rows + tt - 1) / tt : 0, nt = min((per + 31) & ~31, 256);  // tokens of a tile
   const int tiles = a.pair_units * tt, items = nt * tt >= rows ? tiles * S : 0;
@@ -284,14 +283,10 @@ cudaError_t launch_mid(const MidPlan& p, int* err, cudaStream_t stream) {
   }
   MidArgs a;
   a.f.nkb = p.K / MD_BK;
-  a.f.nt_max = 0;
-  a.f.units = 0;
-  a.f.tiles = 0;
   a.f.N = p.N;
   a.f.M = p.M;
   a.f.ep = p.ep;
   a.shapes = p.shapes;
-  a.shape = p.shape;
   a.pair_units = p.N / 256;
   a.flags = p.flags;
   cudaLaunchConfig_t cfg = {};
@@ -359,14 +354,12 @@ cudaError_t mid_plan(MidPlan* p, const void* X, int M, int K, const void* W, int
   p->epi = epi;
   p->ep = ep;
   p->grid = num_sms / 2 * 2;
-  const MidShape s = mid_shape(M, N, K, epi, num_sms / 2);
-  p->shape = s.tt + 256 * s.splits;
   p->flags_needed = (size_t)(N / 256) * ((M + 255) / 256 + MD_MORE_TILES) * 2;
   return cudaSuccess;
 }
 
 cudaError_t mid_launch(const MidPlan& p, int* err, cudaStream_t stream) {
-  if (!p.flags) return cudaErrorInvalidValue;
+  if (!p.flags || !p.shapes) return cudaErrorInvalidValue;
   switch (p.epi) {
     case EPI_RESID_F32: return launch_mid<EPI_RESID_F32>(p, err, stream);
     case EPI_QKV_ROPE: return launch_mid<EPI_QKV_ROPE>(p, err, stream);
