@@ -1,7 +1,7 @@
 """The few-row GEMM (at most 128 rows; weight rows on the MMA's M side) against an fp32
 reference of the same bf16 operands, at the edges of its tiles: row counts around the 32-row
 groups, output widths around the 128-row weight tiles, K from one 64-wide block to a depth at
-which every weight tile is cut over several SMs and summed from partials.
+which every weight tile is cut over the CTAs of a cluster.
 
 Tolerances.  Both sides multiply the same bf16 values; a product is exact in fp32, so they
 differ by fp32 rounding in K-term sums, at most K * 2^-24 * sum |a w| per element (taken as
@@ -50,7 +50,7 @@ def test_repeats_bit_for_bit(ctx):
     a, w, _, _ = _operands(96, 4096, 4096, 5)
     first = torch.empty(96, 4096, dtype=torch.bfloat16, device="cuda")
     ctx.op_linear(a, w, first)
-    for _ in range(20):  # which CTA completes a cut tile varies, its sum does not
+    for _ in range(20):  # (a cut tile's sums are added in K order)
         out = torch.empty_like(first)
         ctx.op_linear(a, w, out)
         assert torch.equal(out.view(torch.int16), first.view(torch.int16))
