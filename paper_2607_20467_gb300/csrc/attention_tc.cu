@@ -74,9 +74,10 @@ struct AttnUnit {
   int row[8], col[8];
 };
 // How a launch's rows are cut: bands per unit; whether the keys of a unit are split over the
-// cluster, and this CTA's key blocks [jb, jb + n).  dead: a wait of this CTA has run out.
+// cluster, and this CTA's key blocks [jb, jb + n).  dead: a wait of this CTA has run out.  b0,
+// before: the 32 sequences that the last unit was found in, and the units of those before them.
 struct AttnLaunch {
-  int bands, split, jb, n, dead;
+  int bands, split, jb, n, dead, b0, before;
 };
 
 template <int HD>
@@ -297,7 +298,8 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         len = q_rows;
       }
     } else {  // rows [seq_off, seq_off + seq_len) of q and of the output
-      for (int b0 = 0, before = 0; b0 < B; b0 += 32) {
+      int b0 = launch.b0, before = launch.before;  // (a CTA's units come in order)
+      for (; b0 < B; b0 += 32) {
         const bool is = b0 + lane < B;
         const int n = is ? seq_len[b0 + lane] : 0, o = is ? seq_off[b0 + lane] : 0, own = attn_units(n, rep, cut);
         int upto = own;
@@ -316,6 +318,11 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
           break;
         }
         before += __shfl_sync(0xffffffffu, upto, 31);
+      }
+      __syncwarp();
+      if (lane == 0) {
+        launch.b0 = b0;
+        launch.before = before;
       }
     }
     AttnUnit& u = units[it & 1];
@@ -358,7 +365,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
         launch.split = keys;
         launch.jb = keys ? rank * nb >> sh : 0;
         launch.n = (keys ? (rank + 1) * nb >> sh : nb) - launch.jb;
-        launch.dead = 0;
+        launch.dead = launch.b0 = launch.before = 0;
       }
       __syncwarp();
     };
