@@ -209,13 +209,14 @@ __global__ void __launch_bounds__(MD_THREADS, 1)
     // ------------------------------------------------ epilogue warps 2..5 (both CTAs)
     const int q = warp & 3;  // TMEM lane quarter: weight rows 32 q .. 32 q + 31 of this CTA's 128
     const int et = (int)threadIdx.x - 64;
+    bool ok = true;  // (after a failed wait a warp still meets the others at every barrier of its items)
     MidItem it;
     for (int idx = 0; item(idx, it); ++idx) {
       const int ab = idx & 1;
-      if (!epilogue_wait(tfull0 + 8 * ab, (uint32_t)(idx >> 1) & 1u, abort_flag)) {
+      if (ok && !__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * ab, (uint32_t)(idx >> 1) & 1u, abort_flag))) {
+        ok = false;
         *abort_flag = 1;
         report_error(err, DERR_WAIT_TIMEOUT);
-        break;
       }
       tc_fence_after();
       const int tok0 = it.tk * nt, n = min(nt, rows - tok0), u = 2 * it.u2 + rank;
@@ -234,12 +235,14 @@ __global__ void __launch_bounds__(MD_THREADS, 1)
           pos_s[et] = a.f.ep.row_pos[tok0 + t0 + et];
           seq_s[et] = a.f.ep.row_seq[tok0 + t0 + et];
         }
-        uint32_t v[32];
-        tmem_ld32(taddr + (uint32_t)t0, v);
-        tmem_ld_wait();
-        const uint32_t at = stg + (uint32_t)(q * 32 + lane) * 4;
+        if (ok) {
+          uint32_t v[32];
+          tmem_ld32(taddr + (uint32_t)t0, v);
+          tmem_ld_wait();
+          const uint32_t at = stg + (uint32_t)(q * 32 + lane) * 4;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) st_shared_f32(at + (uint32_t)(i * FW_PITCH * 4), f32(v[i]));
+          for (int i = 0; i < 32; ++i) st_shared_f32(at + (uint32_t)(i * FW_PITCH * 4), f32(v[i]));
+        }
         if (t0 + MD_CHUNK >= n) {  // the accumulator has been read
           tc_fence_before();
           __syncwarp();

@@ -1245,19 +1245,20 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
     o.box0 = stg + (uint32_t)(q * 2 * BOX_BYTES);
     o.lane = lane;
     o.n = 0;
+    // After a failed wait a warp does no more work, but meets the others at every barrier of its items
+    // (a vote of the warps on each item instead cost a QKV launch of 96 tiles 0.65 us, and a fused
+    // MLP of d 768, ffn 2048 on 8192 rows 2.5 of 62 us)
+    bool ok = true;
     Item it;
     for (int idx = 0; next_item(idx, sc, cluster, it); ++idx) {
       const int ab = idx & 1;
       const uint32_t aph = (uint32_t)(idx >> 1) & 1u;
-      // (with the DSMEM split no item passes a barrier of the epilogue: each warp goes on by itself.
-      // Waiting for one another cost a QKV launch of 96 tiles 0.65 us)
-      const bool there = DS ? __all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * ab, aph, abort_flag)) != 0
-                            : epilogue_wait(tfull0 + 8 * ab, aph, abort_flag);
-      if (!there) {
+      if (ok && !__all_sync(0xffffffffu, mbar_wait(tfull0 + 8 * ab, aph, abort_flag))) {
+        ok = false;
         *abort_flag = 1;
         report_error(err, DERR_WAIT_TIMEOUT);
-        break;
       }
+      if (DS && !ok) break;  // (no barriers there)
       tc_fence_after();
       int m_blk, n_blk;
       tile_mn(it.t, m_blk, n_blk);
@@ -1269,7 +1270,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
       s.taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * 256);
       s.row = row_local;
       if (it.kind == IT_PLAIN) {
-        epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep, it.piece, it.width);
+        if (ok) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep, it.piece, it.width);
         if (FUSE) {
           // publish the tile's act columns to the second GEMM's items that read them: once
           // this CTA's stores have completed, one arrival per split range they fall in
@@ -1293,7 +1294,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
           report_error(err, DERR_WAIT_TIMEOUT);
         }
         epilogue_bar();
-        if (!*abort_flag) epilogue_pair<EPI_RESID_F32>(s, o, &tc2, &tmv, &tmk, row, n_blk, M, N2, ep2);
+        if (ok && !*abort_flag) epilogue_pair<EPI_RESID_F32>(s, o, &tc2, &tmv, &tmk, row, n_blk, M, N2, ep2);
         o.drain();
         epilogue_bar();
         if (et == 0) {
@@ -1369,7 +1370,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             report_error(err, DERR_WAIT_TIMEOUT);
           }
           epilogue_bar();
-          if (!*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
+          if (ok && !*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
           o.drain();
           epilogue_bar();
           if (et == 0) {
@@ -1379,7 +1380,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         } else {
           const int S1 = splits - 1;
           if (sp < S1) {
-            store_partial_pair(s, o, &tmw, ((t * S1 + sp) * 2 + (int)rank) * 128 + q * 32);
+            if (ok) store_partial_pair(s, o, &tmw, ((t * S1 + sp) * 2 + (int)rank) * 128 + q * 32);
             o.drain();
             epilogue_bar();
             if (et == 0) {
@@ -1396,7 +1397,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             s.part = ws + ((size_t)t * S1 * 2 + rank) * 128 * 256;
             s.part_stride = (size_t)2 * 128 * 256;
             s.nparts = S1;
-            if (!*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
+            if (ok && !*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
             epilogue_bar();
             if (et == 0) atomicExch(flag, 0);
           }
@@ -1406,7 +1407,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
         int* flag = flags + it.rel * 2 + rank;
         const int y_slot0 = ((it.rel * ws_slots) * 2 + (int)rank) * 128 + q * 32;
         if (it.kind == IT_PART) {
-          store_partial_pair(s, o, &tmw, y_slot0 + it.slot * 256);
+          if (ok) store_partial_pair(s, o, &tmw, y_slot0 + it.slot * 256);
           o.drain();
           epilogue_bar();
           if (et == 0) {
@@ -1419,7 +1420,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
             report_error(err, DERR_WAIT_TIMEOUT);
           }
           epilogue_bar();
-          if (it.slot > 0 && !*abort_flag) {
+          if (ok && it.slot > 0 && !*abort_flag) {
             const uint32_t tsum = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((ab ^ 1) * 256);
             if (fixup_to_tmem(&tmw, y_slot0, 256, it.slot, base + (uint32_t)(q * (RING2_BYTES / 4)),
                               fix0 + (uint32_t)(q * 8 * FIX_BOXES), tsum, lane, abort_flag, err)) {
@@ -1427,7 +1428,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1)
               s.tsum = tsum;
             }
           }
-          if (!*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
+          if (ok && !*abort_flag) epilogue_pair<EPI>(s, o, &tmc, &tmv, &tmk, row, n_blk, M, N, ep);
           epilogue_bar();
           if (et == 0) atomicExch(flag, 0);
         }

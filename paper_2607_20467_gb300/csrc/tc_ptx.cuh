@@ -366,19 +366,6 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
 __device__ __forceinline__ void epilogue_bar() {  // the 128 epilogue threads (warps 2..5)
   asm volatile("bar.sync 1, 128;" ::: "memory");
 }
-// mbar_wait with one outcome for all 128 epilogue threads, whichever of them saw it fail (after an
-// abort a thread's poll may fall before or after the signal): they meet at the same barriers, so
-// either all of them leave a loop or none does, and a warp reads TMEM whole.
-__device__ __noinline__ bool epilogue_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  uint32_t ok = __all_sync(0xffffffffu, mbar_wait_inline(bar, parity, abort_flag));
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %0, 0;\n\t"
-      "bar.red.and.pred q, 1, 128, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}\n"
-      : "+r"(ok)::"memory");
-  return ok != 0;
-}
 // On the way out of an aborted CTA of a pair: the copies in flight to its shared memory land
 // (microseconds) before that goes to another block.  By time, as they complete on a barrier of
 // the pair's leader, which an abort may leave without its own arrival, so that it never flips.
